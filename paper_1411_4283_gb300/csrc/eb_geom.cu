@@ -186,6 +186,13 @@ __device__ __forceinline__ void mon2(int i, int* p0, int* p1) {
   *p1 = i;
 }
 
+// a^2 - b^2 with its two roundings fixed (the square of b exact: sq_less, of a exact: sq_over).  Positions in a
+// cell come from square roots of such differences of squares of size (R/h)^2, so the moments of a cell of tiny
+// volume or area hold their last bits: left to the compiler's contraction, they would change with the code
+// around them (1e-11 of the patch moments and 4e-8 of a volume fraction of 1e-13 at 63^3).
+__device__ __forceinline__ double sq_less(double a, double b) { return fma(-b, b, __dmul_rn(a, a)); }
+__device__ __forceinline__ double sq_over(double a, double b) { return fma(a, a, -__dmul_rn(b, b)); }
+
 // fluid intervals of the segment [-1/2, 1/2] of a line at signed distance dn from the circle centre, with
 // the circle's chord at tangential position ct: outside fluid keeps the segment minus the chord,
 // inside fluid the segment's part within it.  Returns the count (<= 2).
@@ -758,7 +765,7 @@ __device__ int square_arcs(double cx, double cy, double rho, double* a0, double*
   int na = 0;
   for (int s = -1; s <= 1; s += 2) {
     const double e = 0.5 * s;
-    double d2 = rho * rho - (e - cx) * (e - cx);
+    double d2 = sq_over(rho, e - cx);
     if (d2 >= 0.0) {
       const double w = sqrt(d2);
       for (int u = -1; u <= 1; u += 2) {
@@ -766,7 +773,7 @@ __device__ int square_arcs(double cx, double cy, double rho, double* a0, double*
         if (yy >= -0.5 && yy <= 0.5) ang[na++] = atan2(yy - cy, e - cx);
       }
     }
-    d2 = rho * rho - (e - cy) * (e - cy);
+    d2 = sq_over(rho, e - cy);
     if (d2 >= 0.0) {
       const double w = sqrt(d2);
       for (int u = -1; u <= 1; u += 2) {
@@ -807,13 +814,23 @@ __device__ __forceinline__ void sin2_node(const GlRuleT& gl, int g, double a, do
   *w = 0.5 * gl.w[g] * (b - a) * M_PI * sn * cs;
 }
 
-// The rules of the moment kernels, with what depends on the node alone worked out on the host: the
-// sin^2-mapped panel nodes (t = a + (b - a) pos, weight (b - a) wt) and Gauss-Legendre rules of 8, 10 and
-// 12 points for the arcs (the positive nodes; the rules are symmetric).
+// The rules of the moment kernels: the sin^2-mapped panel nodes of sin2_node (a block turns the Gauss-Legendre
+// nodes into the sines of sin2_node, and the weights into its weights over b - a, once: panel_rule) and
+// Gauss-Legendre rules of 8, 10 and 12 points for the arcs (the positive nodes; the rules are symmetric).
 struct PatchRule {
   double pos[GEO_GLT], wt[GEO_GLT];
   double ax[15], aw[15];  // rules of 8 (4 pairs, at 0), 10 (5, at 4) and 12 points (6, at 9)
 };
+
+__device__ __forceinline__ void panel_rule(const PatchRule& rule, double* pos, double* wt) {
+  for (int g = threadIdx.x; g < GEO_GLT; g += blockDim.x) {
+    const double s = 0.5 * rule.pos[g] + 0.5;
+    const double sn = sin(0.5 * M_PI * s), cs = cos(0.5 * M_PI * s);
+    pos[g] = sn;
+    wt[g] = 0.5 * rule.wt[g] * M_PI * sn * cs;
+  }
+}
+__device__ __forceinline__ double panel_node(double a, double width, double sn) { return a + width * sn * sn; }
 
 // Points for an arc piece of half-angle hw.  The integrand is a product of at most six factors x, y and
 // cos or sin of the angle, with |x|, |y| <= 1/2: its Taylor coefficient of degree 2n in the angle over hw is
@@ -880,6 +897,8 @@ __global__ void __launch_bounds__(PATCH_WARPS * 32) k_sphere_patch(Spheres B, co
   for (int i = threadIdx.x; i < (int)(sizeof(PatchRule) / 8); i += blockDim.x)
     reinterpret_cast<double*>(&ru)[i] = reinterpret_cast<const double*>(&rule)[i];
   __syncthreads();
+  panel_rule(rule, ru.pos, ru.wt);
+  __syncthreads();
   const int64_t t = (int64_t)blockIdx.x * PATCH_WARPS + warp;
   if (t >= n) return;
   const int c = cells[t];
@@ -903,7 +922,9 @@ __global__ void __launch_bounds__(PATCH_WARPS * 32) k_sphere_patch(Spheres B, co
       const bool corner = lane >= 10;
       const int j = corner ? lane - 10 : lane - 2;  // bit 0: edge, bit 1: axis or the other edge, bit 2: side
       const double ex = ((j & 1) ? 0.5 : -0.5) - cx, ey = (((corner ? j >> 1 : j) & 1) ? 0.5 : -0.5) - cy;
-      const double qq = R * R - (corner || !(j & 2) ? ex * ex : 0.0) - (corner || (j & 2) ? ey * ey : 0.0);
+      const double e1 = corner || !(j & 2) ? ex : ey;
+      double qq = sq_less(R, e1);
+      if (corner) qq = __dsub_rn(qq, __dmul_rn(ey, ey));
       z = cz + ((j & 4) ? 1.0 : -1.0) * sqrt(fmax(qq, 0.0));
       valid = qq > 0.0 && z > zl && z < zh;
     }
@@ -953,7 +974,7 @@ __global__ void __launch_bounds__(PATCH_WARPS * 32) k_sphere_patch(Spheres B, co
       const int pn = M.panel[(i0 + lane) / GEO_GLT], gz = (i0 + lane) % GEO_GLT;
       const double ta = M.br[pn], tw = M.br[pn + 1] - ta;
       double sth, cth;
-      sincos(ta + tw * ru.pos[gz], &sth, &cth);
+      sincos(panel_node(ta, tw, ru.pos[gz]), &sth, &cth);
       const double rho = R * sth;
       ez = R * cth;
       z = cz + ez;
@@ -1043,99 +1064,39 @@ __global__ void __launch_bounds__(PATCH_WARPS * 32) k_sphere_patch(Spheres B, co
 }
 
 // (+-1/2)^e
-__device__ constexpr double half_pow(int sign, int e) {
+__host__ __device__ constexpr double half_pow(int sign, int e) {
   double r = 1.0;
   for (int i = 0; i < e; ++i) r *= sign < 0 ? -0.5 : 0.5;
   return r;
 }
 
-// the moments of all the faces the sphere cuts, before the ends are settled (k_sphere_faces)
-struct RawFaces {
-  const uint8_t* flag[3];
-  const int64_t* pos[3];     // place of a cut face in its direction's list
-  const double* mom[3];
+// Moments int u^a v^b over the fluid part of the square [-1/2,1/2]^2 of a plane the sphere cuts in the disk
+// (cu, cv, rho) (rho <= 0: no disk), by a warp: the sin^2-mapped nodes of the u-panels over the lanes, then
+// one sum over the warp (in every lane).  Outside a sphere the full columns beyond the disk's u-range come in
+// closed form and the parts of a column beyond the chord node by node (a nearly closed face is not the small
+// difference of the square and the disk).
+struct DiskSmem {
+  double pos[GEO_GLT], wt[GEO_GLT], br[4][8];
 };
-
-// volume moments from the patch part and the fluid parts of the two faces normal to the divergence
-// direction (thread per cell and monomial): those faces' moments are in the face tables already, a face
-// the sphere does not reach is covered or full
-__global__ void k_sphere_vol(Spheres B, int N, double h, const int32_t* __restrict__ cells, int64_t n,
-                             const int32_t* __restrict__ cbody, int q, int K, RawFaces f,
-                             const double* __restrict__ volp, double* vol) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n * K) return;
-  const int64_t t = i / K;
-  const int c = cells[t];
-  const int x[3] = {c % N, (c / N) % N, c / (N * N)};
-  const int b = cbody[c];
-  const double cx = (B.c[b][0] - (x[0] + 0.5) * h) / h, cy = (B.c[b][1] - (x[1] + 0.5) * h) / h;
-  const double cz = (B.c[b][2] - (x[2] + 0.5) * h) / h;
-  // the direction most tangent to the patch (as in k_sphere_patch) and the two faces normal to it
-  const int dd = (fabs(cx) <= fabs(cy) && fabs(cx) <= fabs(cz)) ? 0 : (fabs(cy) <= fabs(cz) ? 1 : 2);
-  const int u = dd == 0 ? 1 : 0, v = dd == 2 ? 1 : 2;
-  int p[3];
-  mon3((int)(i % K), p);
-  const int k2 = idx2(p[u], p[v]), K2 = (q + 1) * (q + 2) / 2;
-  const int m0 = N + (dd == 0), m1 = N + (dd == 1);
-  double acc = volp[i];
-  for (int s = 0; s < 2; ++s) {
-    const int64_t fi = (x[0] + (dd == 0 && s)) + (int64_t)m0 * ((x[1] + (dd == 1 && s)) + (int64_t)m1 * (x[2] + (dd == 2 && s)));
-    const int fl = f.flag[dd][fi];
-    double fm = 0.0;
-    if (fl == 2) fm = f.mom[dd][f.pos[dd][fi] * K2 + k2];
-    else if (fl == 1 && !(p[u] & 1) && !(p[v] & 1))
-      fm = half_pow(1, p[u] + p[v]) / ((p[u] + 1) * (p[v] + 1));
-    acc += (s ? 1.0 : -1.0) * half_pow(s ? 1 : -1, p[dd] + 1) * fm;
-  }
-  vol[i] = acc / (p[dd] + 1);
-}
-
-// Tangential moments of the cut faces normal to dir, int u^a v^b over the fluid part of the square the
-// sphere cuts in the disk (cu, cv, rho): a warp per face, the sin^2-mapped nodes of the u-panels over the
-// lanes, then one sum over the warp.  Outside a sphere the full columns beyond the disk's u-range come in
-// closed form and the parts of a column beyond the chord node by node (a nearly closed face is not the
-// small difference of the square and the disk).  FP64 issue bound; a thread per face took 3.3 ms for a
-// direction of the 96^3 box minus a sphere (a chain of one thread's nodes), this 0.34 ms.
 template <int Q>
-__global__ void __launch_bounds__(128) k_sphere_faces(Spheres B, const __grid_constant__ PatchRule rule, int N, int dir,
-                                                      double h, const int32_t* __restrict__ faces, int64_t n,
-                                                      const int32_t* __restrict__ fbody, double* out) {
+__device__ __forceinline__ void disk_square(double cu, double cv, double rho, bool inside, DiskSmem& S,
+                                            double (&acc)[(Q + 1) * (Q + 2) / 2]) {
   constexpr int K2 = (Q + 1) * (Q + 2) / 2;
-  __shared__ double pos[GEO_GLT], wt[GEO_GLT], brs[4][8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < GEO_GLT; i += blockDim.x) {
-    pos[i] = rule.pos[i];
-    wt[i] = rule.wt[i];
-  }
-  __syncthreads();
-  const int64_t t = (int64_t)blockIdx.x * 4 + warp;
-  if (t >= n) return;
-  const int f = faces[t];
-  const int m0 = N + (dir == 0), m1 = N + (dir == 1);
-  const int i3[3] = {f % m0, (f / m0) % m1, f / (m0 * m1)};
-  const int b = fbody[f];
-  const int u = dir == 0 ? 1 : 0, v = dir == 2 ? 1 : 2;  // tangential dims, ascending
-  const double dn = (i3[dir] * h - B.c[b][dir]) / h;
-  const double cu = (B.c[b][u] - (i3[u] + 0.5) * h) / h, cv = (B.c[b][v] - (i3[v] + 0.5) * h) / h;
-  const double R = B.r[b] / h, d2 = R * R - dn * dn;
-  const double rho = d2 > 0.0 ? sqrt(d2) : 0.0;
   const double lo = fmax(-0.5, cu - rho), hi = fmin(0.5, cu + rho);
   const bool disk = rho > 0.0 && hi > lo;
-  double acc[K2];
 #pragma unroll
   for (int k = 0; k < K2; ++k) acc[k] = 0.0;
   if (disk) {
-    // breakpoints, one candidate per lane: the range ends and where the circle meets v = +-1/2 (shifted by
-    // 1/2 to be non-negative for the sort)
+    // breakpoints, one candidate per lane: the range ends and where the circle meets v = +-1/2
     double uu = lane == 0 ? lo : hi;
     bool valid = lane < 2;
     if (lane >= 2 && lane < 6) {
       const double dv = ((lane & 1) ? 0.5 : -0.5) - cv;
-      const double w2 = rho * rho - dv * dv;
-      uu = cu + ((lane & 2) ? -1.0 : 1.0) * sqrt(fmax(w2, 0.0));
+      uu = cu + ((lane & 2) ? -1.0 : 1.0) * sqrt(fmax(sq_less(rho, dv), 0.0));
       valid = fabs(dv) < rho && uu > lo && uu < hi;
     }
-    double* br = brs[warp];
+    double* br = S.br[warp];
     const unsigned m = __ballot_sync(0xffffffffu, valid);
     int rank = 0;
     for (unsigned r = m; r; r &= r - 1) {
@@ -1143,21 +1104,22 @@ __global__ void __launch_bounds__(128) k_sphere_faces(Spheres B, const __grid_co
       const double o = __shfl_sync(0xffffffffu, uu, j);
       rank += o < uu || (o == uu && j < lane);
     }
+    __syncwarp();  // the warp's last use of br
     if (valid) br[rank] = uu;
     __syncwarp();
     const int total = (__popc(m) - 1) * GEO_GLT;
     for (int i = lane; i < total; i += 32) {
       const double a = br[i / GEO_GLT], pw = br[i / GEO_GLT + 1] - a;
       if (!(pw > 0.0)) continue;
-      const double uq = a + pw * pos[i % GEO_GLT], wu = pw * wt[i % GEO_GLT];
-      const double hw = sqrt(fmax(rho * rho - (uq - cu) * (uq - cu), 0.0));
+      const double uq = panel_node(a, pw, S.pos[i % GEO_GLT]), wu = pw * S.wt[i % GEO_GLT];
+      const double du = uq - cu, hw = sqrt(fmax(sq_less(rho, du), 0.0));
       const double va = fmin(fmax(cv - hw, -0.5), 0.5), vb = fmin(fmax(cv + hw, -0.5), 0.5);
       double pa = va, pb = vb, vp[Q + 1], up[Q + 1];
 #pragma unroll
       for (int k = 0; k <= Q; ++k) {
         // the chord, or the two parts of the column beyond it
         const double full = half_pow(1, k + 1), rk = 1.0 / (k + 1);
-        const double s = B.inside ? pb - pa : (pa - ((k & 1) ? full : -full)) + (full - pb);
+        const double s = inside ? pb - pa : (pa - ((k & 1) ? full : -full)) + (full - pb);
         vp[k] = s * (wu * rk);
         pa *= va;
         pb *= vb;
@@ -1172,7 +1134,7 @@ __global__ void __launch_bounds__(128) k_sphere_faces(Spheres B, const __grid_co
     for (int k = 0; k < K2; ++k)
       for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
   }
-  if (!B.inside) {  // the columns beyond the disk's u-range
+  if (!inside) {  // the columns beyond the disk's u-range
     double ua[2] = {-0.5, hi}, ub[2] = {disk ? lo : 0.5, 0.5};
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -1189,9 +1151,93 @@ __global__ void __launch_bounds__(128) k_sphere_faces(Spheres B, const __grid_co
       }
     }
   }
+}
+
+__device__ __forceinline__ void disk_rule(const PatchRule& rule, DiskSmem& S) {
+  panel_rule(rule, S.pos, S.wt);
+  __syncthreads();
+}
+
+// Volume moments from the patch part and the fluid parts of the two faces normal to the divergence direction
+// (a warp per cell).  Those faces' moments are integrated here once more, from the cell's own coordinates: the
+// volume of a small cell is the difference of these terms, and its relative error the rounding of their
+// coordinates.
+template <int Q>
+__global__ void __launch_bounds__(128) k_sphere_vol(Spheres B, const __grid_constant__ PatchRule rule, int N, double h,
+                                                    const int32_t* __restrict__ cells, int64_t n,
+                                                    const int32_t* __restrict__ cbody, const double* __restrict__ volp,
+                                                    double* vol) {
+  constexpr int K = (Q + 1) * (Q + 2) * (Q + 3) / 6, K2 = (Q + 1) * (Q + 2) / 2;
+  __shared__ DiskSmem S;
+  __shared__ double fms[4][K2];
+  disk_rule(rule, S);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t t = (int64_t)blockIdx.x * 4 + warp;
+  if (t >= n) return;
+  const int c = cells[t];
+  const int ix = c % N, iy = (c / N) % N, iz = c / (N * N);
+  const int b = cbody[c];
+  const double cx = (B.c[b][0] - (ix + 0.5) * h) / h, cy = (B.c[b][1] - (iy + 0.5) * h) / h;
+  const double cz = (B.c[b][2] - (iz + 0.5) * h) / h, R = B.r[b] / h;
+  // the direction most tangent to the patch (as in k_sphere_patch) and the two faces normal to it
+  const int dd = (fabs(cx) <= fabs(cy) && fabs(cx) <= fabs(cz)) ? 0 : (fabs(cy) <= fabs(cz) ? 1 : 2);
+  const double cd = dd == 0 ? cx : (dd == 1 ? cy : cz), cu = dd == 0 ? cy : cx, cv = dd == 2 ? cy : cz;
+  double acc[(K + 31) / 32];
+#pragma unroll
+  for (int i = 0; i < (K + 31) / 32; ++i) acc[i] = lane + 32 * i < K ? volp[t * K + lane + 32 * i] : 0.0;
+  for (int s = -1; s <= 1; s += 2) {
+    const double xe = 0.5 * s, d2 = sq_less(R, xe - cd);
+    double fm[K2];
+    disk_square<Q>(cu, cv, d2 > 0.0 ? sqrt(d2) : 0.0, B.inside, S, fm);
+    if (lane == 0) {
+#pragma unroll
+      for (int k = 0; k < K2; ++k) fms[warp][k] = fm[k];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < (K + 31) / 32; ++i) {
+      if (lane + 32 * i >= K) continue;
+      int p[3];
+      mon3(lane + 32 * i, p);
+      const int pu = dd == 0 ? p[1] : p[0], pv = dd == 2 ? p[1] : p[2];
+      acc[i] += s * half_pow(s, p[dd] + 1) * fms[warp][idx2(pu, pv)];
+    }
+    __syncwarp();
+  }
+#pragma unroll
+  for (int i = 0; i < (K + 31) / 32; ++i) {
+    if (lane + 32 * i >= K) continue;
+    int p[3];
+    mon3(lane + 32 * i, p);
+    vol[t * K + lane + 32 * i] = acc[i] / (p[dd] + 1);
+  }
+}
+
+// Tangential moments of the cut faces normal to dir (a warp per face).  FP64 issue bound; a thread per face
+// took 3.3 ms for a direction of the 96^3 box minus a sphere (a chain of one thread's nodes), this 0.34 ms.
+template <int Q>
+__global__ void __launch_bounds__(128) k_sphere_faces(Spheres B, const __grid_constant__ PatchRule rule, int N, int dir,
+                                                      double h, const int32_t* __restrict__ faces, int64_t n,
+                                                      const int32_t* __restrict__ fbody, double* out) {
+  constexpr int K2 = (Q + 1) * (Q + 2) / 2;
+  __shared__ DiskSmem S;
+  disk_rule(rule, S);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t t = (int64_t)blockIdx.x * 4 + warp;
+  if (t >= n) return;
+  const int f = faces[t];
+  const int m0 = N + (dir == 0), m1 = N + (dir == 1);
+  const int i3[3] = {f % m0, (f / m0) % m1, f / (m0 * m1)};
+  const int b = fbody[f];
+  const int u = dir == 0 ? 1 : 0, v = dir == 2 ? 1 : 2;  // tangential dims, ascending
+  const double dn = (i3[dir] * h - B.c[b][dir]) / h;
+  const double cu = (B.c[b][u] - (i3[u] + 0.5) * h) / h, cv = (B.c[b][v] - (i3[v] + 0.5) * h) / h;
+  const double R = B.r[b] / h, d2 = sq_over(R, dn);
+  double fm[K2];
+  disk_square<Q>(cu, cv, d2 > 0.0 ? sqrt(d2) : 0.0, B.inside, S, fm);
   if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < K2; ++k) out[t * K2 + k] = acc[k];
+    for (int k = 0; k < K2; ++k) out[t * K2 + k] = fm[k];
   }
 }
 
@@ -1609,9 +1655,8 @@ cudaError_t geo_scan(const int32_t* sel, int64_t n, int64_t* pos, int64_t* total
   return cudaStreamSynchronize(A.s);
 }
 
-// list of the indices i < n with flag[i] == v, ascending (a temporary), and each one's place in it (pos)
-cudaError_t geo_list(const uint8_t* flag, int64_t n, uint8_t v, int32_t** list, int64_t* count, GeoAlloc& A,
-                     int64_t** pos_out = nullptr) {
+// list of the indices i < n with flag[i] == v, ascending (a temporary)
+cudaError_t geo_list(const uint8_t* flag, int64_t n, uint8_t v, int32_t** list, int64_t* count, GeoAlloc& A) {
   int32_t* sel;
   int64_t* pos;
   cudaError_t e;
@@ -1620,20 +1665,18 @@ cudaError_t geo_list(const uint8_t* flag, int64_t n, uint8_t v, int32_t** list, 
   eb::count_launch();
   if ((e = geo_scan(sel, n, pos, count, A))) return e;
   if ((e = A.temp(list, *count))) return e;
-  if (pos_out) *pos_out = pos;
   k_geo_compact<<<nb256(n), 256, 0, A.s>>>(sel, pos, n, *list);
   eb::count_launch();
   return cudaGetLastError();
 }
 
-// the rules of the sphere kernels: the sin^2 map of sin2_node and the arc rules of arc_rule
+// the rules of the sphere kernels
 PatchRule patch_rule() {
   PatchRule r;
   const GlRuleT t = gl_rule<GEO_GLT>();
   for (int g = 0; g < GEO_GLT; ++g) {
-    const double a = 0.5 * M_PI * (0.5 * t.x[g] + 0.5);
-    r.pos[g] = sin(a) * sin(a);
-    r.wt[g] = 0.5 * t.w[g] * M_PI * sin(a) * cos(a);
+    r.pos[g] = t.x[g];
+    r.wt[g] = t.w[g];
   }
   const auto g8 = gl_rule<8>();
   const auto g10 = gl_rule<10>();
@@ -1666,6 +1709,20 @@ cudaError_t sphere_patch_launch(int q, const Spheres& B, const PatchRule& rule, 
     case 3: return patch_launch<3>(B, rule, N, h, cells, n, cbody, eb, ebn, volp, s);
     default: return patch_launch<4>(B, rule, N, h, cells, n, cbody, eb, ebn, volp, s);
   }
+}
+
+cudaError_t sphere_vol_launch(int q, const Spheres& B, const PatchRule& rule, int N, double h, const int32_t* cells,
+                              int64_t n, const int32_t* cbody, const double* volp, double* vol, cudaStream_t s) {
+  const unsigned nb = (unsigned)((n + 3) / 4);
+  switch (q) {
+    case 0: k_sphere_vol<0><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol); break;
+    case 1: k_sphere_vol<1><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol); break;
+    case 2: k_sphere_vol<2><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol); break;
+    case 3: k_sphere_vol<3><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol); break;
+    default: k_sphere_vol<4><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol); break;
+  }
+  eb::count_launch();
+  return cudaGetLastError();
 }
 
 cudaError_t sphere_faces_launch(int q, const Spheres& B, const PatchRule& rule, int N, int dir, double h,
@@ -1925,23 +1982,18 @@ extern "C" eb_status eb_geometry_spheres(int32_t N, int32_t n_body, const double
       k_geo_classify3<<<nb256(nf), 256, 0, s>>>(B, N, h, d, nf, ff[d], fbody[d], err);
       eb::count_launch();
     }
-    // the cut faces' moments first: the cut cells' volumes use them
+    // all lists before the moments: one wait for the classification's result
     int32_t* cf0[3];
     int64_t nf0[3];
     double* fm0[3];
-    RawFaces raw;
     {
       int32_t* cut0;
       int64_t nc0 = 0;
       GEO_TRY(geo_list(cflag, ncell, 2, &cut0, &nc0, A));
       for (int d = 0; d < 3; ++d) {
         const int64_t nf = (int64_t)(N + (d == 0)) * (N + (d == 1)) * (N + (d == 2));
-        int64_t* fpos;
-        GEO_TRY(geo_list(ff[d], nf, 2, &cf0[d], &nf0[d], A, &fpos));
+        GEO_TRY(geo_list(ff[d], nf, 2, &cf0[d], &nf0[d], A));
         GEO_TRY(A.temp(&fm0[d], nf0[d] * KF));
-        raw.flag[d] = ff[d];
-        raw.pos[d] = fpos;
-        raw.mom[d] = fm0[d];
       }
       int32_t herr = 0;
       GEO_TRY(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, s));
@@ -1960,8 +2012,7 @@ extern "C" eb_status eb_geometry_spheres(int32_t N, int32_t n_body, const double
         if (nf0[d] > 0) GEO_TRY(sphere_faces_launch(q, B, rule, N, d, h, cf0[d], nf0[d], fbody[d], fm0[d], s));
       if (nc0 > 0) {
         GEO_TRY(sphere_patch_launch(q, B, rule, N, h, cut0, nc0, cbody, eb0, ebn0, volp, s));
-        k_sphere_vol<<<nb256(nc0 * K), 256, 0, s>>>(B, N, h, cut0, nc0, cbody, q, K, raw, volp, vol0);
-        eb::count_launch();
+        GEO_TRY(sphere_vol_launch(q, B, rule, N, h, cut0, nc0, cbody, volp, vol0, s));
       }
       int32_t* keep;
       int64_t* pos;

@@ -591,7 +591,7 @@ struct BuildCtx {
   eb_build_info* info = nullptr;
   cudaStream_t s = nullptr;
   eb_params P;
-  int R = 0, D = 0, nsm = 0;
+  int R = 0, D = 0, nsm = 0, max_rows = 0;
   int64_t N = 0, n_slots = 0, n_unique = 0;
   Tables T;
   Tables* dT = nullptr;
@@ -1119,12 +1119,12 @@ static eb_status build_pre(BuildCtx& c) {
   ga.cut_of_cell = st->cut_of_cell;
   ga.slot_face = st->slot_face;
   int64_t* counts;
-  int32_t* too_many;
+  int32_t* max_rows;
   EB_TRY(tmp.get(&counts, n_slots + 1));
-  EB_TRY(tmp.get(&too_many, 1));
-  EB_CUDA(cudaMemsetAsync(too_many, 0, 4, s));
+  EB_TRY(tmp.get(&max_rows, 1));
+  EB_CUDA(cudaMemsetAsync(max_rows, 0, 4, s));
   ga.count = counts;
-  ga.too_many = too_many;
+  ga.max_rows = max_rows;
   ga.row_ptr = nullptr;
   k_gather<<<nblk(n_slots, 128), 128, 0, s>>>(ga, n_slots, st->cut_cell); eb::count_launch();
   EB_CUDA(cudaGetLastError());
@@ -1132,10 +1132,9 @@ static eb_status build_pre(BuildCtx& c) {
   int64_t nnz = 0;
   EB_CUDA(cudaMemsetAsync(counts + n_slots, 0, 8, s));
   EB_TRY(scan<int64_t>(counts, n_slots + 1, st->row_ptr, &nnz, s, tmp));
-  int32_t h_too = 0;
-  EB_CUDA(cudaMemcpyAsync(&h_too, too_many, 4, cudaMemcpyDeviceToHost, s));
+  EB_CUDA(cudaMemcpyAsync(&c.max_rows, max_rows, 4, cudaMemcpyDeviceToHost, s));
   EB_CUDA(cudaStreamSynchronize(s));
-  if (h_too) { set_error("a face has more LS rows than the kernel supports"); return EB_ERR_CAPACITY; }
+  if (c.max_rows > MAXROWS) { set_error("a face has more LS rows than the kernel supports"); return EB_ERR_CAPACITY; }
   EB_TRY(dalloc(st, &st->row_desc, nnz));
   EB_TRY(dalloc(st, &st->row_val, nnz));
   ga.row_ptr = st->row_ptr;
@@ -1147,9 +1146,12 @@ static eb_status build_pre(BuildCtx& c) {
   EB_CUDA(cudaGetDevice(&dev));
   EB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   double *ftab, *wtab;
+  float *ftab_h, *ftab_l;
   EB_TRY(tmp.get(&ftab, (size_t)TAB_N * MAXK));
+  EB_TRY(tmp.get(&ftab_h, (size_t)TAB_N * MAXK));
+  EB_TRY(tmp.get(&ftab_l, (size_t)TAB_N * MAXK));
   EB_TRY(tmp.get(&wtab, TAB_N));
-  k_full_rows<<<nblk(TAB_N, 128), 128, 0, s>>>(dm, dT, ftab, wtab); eb::count_launch();
+  k_full_rows<<<nblk(TAB_N, 128), 128, 0, s>>>(dm, dT, ftab, ftab_h, ftab_l, wtab); eb::count_launch();
   int32_t* status;
   EB_TRY(tmp.get(&status, std::max<int64_t>(n_slots, 1)));
   LsArgs& la = c.la;
@@ -1174,6 +1176,8 @@ static eb_status build_pre(BuildCtx& c) {
   la.n_slots = n_slots;
   la.status = status;
   la.ftab = ftab;
+  la.ftab_h = ftab_h;
+  la.ftab_l = ftab_l;
   la.wtab = wtab;
   c.P = P;
   c.R = R;
@@ -1207,9 +1211,14 @@ static eb_status build_ls(BuildCtx* const* cs, int n, cudaStream_t s) {
   auto blocks_for = [&](int64_t systems, int per_cta) {
     return std::max<int64_t>(1, std::min<int64_t>(c0.nsm, (systems + per_cta - 1) / per_cta));
   };
-  const int64_t nb_d = blocks_for(total, LS_SYS), nb_f = blocks_for(total, LS_SYS_F);
-  double* scratch;
-  EB_TRY(tmp.get(&scratch, (size_t)std::max(nb_d * LS_SYS, fp32 ? nb_f * LS_SYS_F : 0) * LS_SCRATCH));
+  int max_rows = 0;
+  for (int i = 0; i < n; ++i) max_rows = std::max(max_rows, cs[i]->max_rows);
+  // FP64 blocks: for every system, or (mixed) sized when the number it left is known
+  double* scratch = nullptr;
+  int64_t mixed_scratch = 0;
+  const int64_t nb_f = fp32 ? lsq_mixed_blocks(c0.T, max_rows, total, c0.nsm, &mixed_scratch) : 0;
+  const int64_t nb_d = fp32 ? 0 : blocks_for(total, LS_SYS);
+  EB_TRY(tmp.get(&scratch, (size_t)(fp32 ? mixed_scratch : nb_d * LS_SYS * LS_SCRATCH)));
   int32_t *next, *lerr, *nfb, *fblist = nullptr;
   double* flops;
   EB_TRY(tmp.get(&next, 1));
@@ -1244,7 +1253,7 @@ static eb_status build_ls(BuildCtx* const* cs, int n, cudaStream_t s) {
   if (total > 0) {
     if (fp32) {
       // FP32 factorisation for every system, then the FP64 one for those it left (status 3)
-      EB_CUDA(lsq_launch(true, (unsigned)nb_f, s, a0, c0.T, n > 1 ? dbatch : nullptr, dbase, n));
+      EB_CUDA(lsq_mixed_launch(nb_f, max_rows, s, a0, c0.T, n > 1 ? dbatch : nullptr, dbase, n));
       eb::count_launch();
       EB_TRY(tmp.get(&fblist, total));
       for (int i = 0; i < n; ++i) {
@@ -1258,11 +1267,13 @@ static eb_status build_ls(BuildCtx* const* cs, int n, cudaStream_t s) {
         EB_CUDA(cudaMemsetAsync(next, 0, 4, s));
         a0.slot_list = fblist;
         a0.n_slots = hn;
-        EB_CUDA(lsq_launch(false, (unsigned)blocks_for(hn, LS_SYS), s, a0, c0.T, n > 1 ? dbatch : nullptr, dbase, n));
+        const int64_t nb = blocks_for(hn, LS_SYS);
+        EB_TRY(tmp.get(&a0.scratch, (size_t)nb * LS_SYS * LS_SCRATCH));
+        EB_CUDA(lsq_launch((unsigned)nb, s, a0, c0.T, n > 1 ? dbatch : nullptr, dbase, n));
         eb::count_launch();
       }
     } else {
-      EB_CUDA(lsq_launch(false, (unsigned)nb_d, s, a0, c0.T, n > 1 ? dbatch : nullptr, dbase, n));
+      EB_CUDA(lsq_launch((unsigned)nb_d, s, a0, c0.T, n > 1 ? dbatch : nullptr, dbase, n));
       eb::count_launch();
     }
   }

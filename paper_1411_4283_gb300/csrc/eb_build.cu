@@ -19,37 +19,9 @@
 #include "eb_internal.cuh"
 #include "eb_tables.cuh"
 #include "eb_build.cuh"
+#include "eb_grid.cuh"
 
 namespace eb {
-
-// ============================================================ geometry helpers
-
-__device__ __forceinline__ void cell_xyz(const Dims& dm, int64_t c, int* x) {
-  x[0] = (int)(c % dm.n[0]);
-  int64_t r = c / dm.n[0];
-  x[1] = (int)(r % dm.n[1]);
-  x[2] = (int)(r / dm.n[1]);
-}
-__device__ __forceinline__ int64_t cell_id(const Dims& dm, const int* x) {
-  return (int64_t)x[0] + (int64_t)dm.n[0] * ((int64_t)x[1] + (int64_t)dm.n[1] * x[2]);
-}
-__device__ __forceinline__ bool in_domain(const Dims& dm, const int* x) {
-  for (int d = 0; d < 3; ++d)
-    if (x[d] < 0 || x[d] >= dm.n[d]) return false;
-  return true;
-}
-// local index of the face normal to d whose coordinates are x (x[d] in 0..n_d)
-__device__ __forceinline__ int64_t face_local(const Dims& dm, int d, const int* x) {
-  int64_t m0 = dm.n[0] + (d == 0), m1 = dm.n[1] + (d == 1);
-  return (int64_t)x[0] + m0 * ((int64_t)x[1] + m1 * x[2]);
-}
-__device__ __forceinline__ void face_xyz(const Dims& dm, int d, int64_t f, int* x) {
-  int64_t m0 = dm.n[0] + (d == 0), m1 = dm.n[1] + (d == 1);
-  x[0] = (int)(f % m0);
-  int64_t r = f / m0;
-  x[1] = (int)(r % m1);
-  x[2] = (int)(r / m1);
-}
 
 // ============================================================ 1. masks and classes
 
@@ -366,7 +338,7 @@ __global__ void k_gather(GatherArgs a, int64_t n_slots, const int32_t* __restric
   else n = gather_rows(a, s, out);
   if (!a.row_ptr) {
     a.count[s] = n;
-    if (n > MAXROWS) atomicExch(a.too_many, 1);
+    if (n > *a.max_rows) atomicMax(a.max_rows, n);
   }
 }
 
@@ -375,23 +347,20 @@ __global__ void k_gather(GatherArgs a, int64_t n_slots, const int32_t* __restric
 __device__ __forceinline__ int tab_index(const double* delta) {
   int i0 = (int)lrint(2.0 * delta[0]) + 11, i1 = (int)lrint(2.0 * delta[1]) + 11, i2 = (int)lrint(2.0 * delta[2]) + 11;
   if (i0 < 0 || i0 >= TAB_S || i1 < 0 || i1 >= TAB_S || i2 < 0 || i2 >= TAB_S) return -1;
-  return i0 + TAB_S * (i1 + TAB_S * i2);
-}
-
-__device__ __forceinline__ double weight_of(const Dims& dm, double r2) {
-  // Sec. 2.4: W_ii = 1 if r < 1/2, else (2r)^-5, r = |x_i - x0| / h
-  if (!dm.weighted || r2 < dm.w_threshold * dm.w_threshold) return 1.0;
-  return pow(4.0 * r2, -0.5 * dm.w_power);
+  const int x[3] = {i0, i1, i2};
+  return tab_place(x);
 }
 
 // Rows of full cells depend only on the offset delta = (cell centre - x0)/h:
 // the average of prod_d xi_d^{p_d} over the unit cell centred at delta is
 // prod_d ((delta_d + 1/2)^{p_d+1} - (delta_d - 1/2)^{p_d+1}) / (p_d + 1).
 __global__ void k_full_rows(Dims dm, const Tables* __restrict__ T, double* __restrict__ ftab,
-                            double* __restrict__ wtab) {
+                            float* __restrict__ ftab_h, float* __restrict__ ftab_l, double* __restrict__ wtab) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= TAB_N) return;
-  double delta[3] = {0.5 * (t % TAB_S - 11), 0.5 * ((t / TAB_S) % TAB_S - 11), 0.5 * (t / (TAB_S * TAB_S) - 11)};
+  constexpr int EVEN = (TAB_S + 1) / 2;  // tab_place's order along x
+  const int tx = t % TAB_S < EVEN ? 2 * (t % TAB_S) : 2 * (t % TAB_S - EVEN) + 1;
+  double delta[3] = {0.5 * (tx - 11), 0.5 * ((t / TAB_S) % TAB_S - 11), 0.5 * (t / (TAB_S * TAB_S) - 11)};
   double oned[3][8];
   for (int d = 0; d < 3; ++d) {
     double a = delta[d] - 0.5, b = delta[d] + 0.5, pa = a, pb = b;
@@ -408,7 +377,10 @@ __global__ void k_full_rows(Dims dm, const Tables* __restrict__ T, double* __res
   for (int i = 0; i < T->K; ++i) {
     double v = 1.0;
     for (int d = 0; d < dm.dim; ++d) v *= oned[d][T->mon[i][d]];
-    ftab[(int64_t)t * MAXK + i] = w * v;
+    v *= w;
+    ftab[(int64_t)i * TAB_N + t] = v;
+    ftab_h[(int64_t)i * TAB_N + t] = (float)v;
+    ftab_l[(int64_t)i * TAB_N + t] = (float)(v - (double)(float)v);
   }
 }
 
@@ -499,8 +471,7 @@ __device__ double row_prepare(const LsArgs& a, const Tables& T, uint32_t desc, c
     }
     int32_t cut = a.cut_of_cell[cid];
     if (kind == 0 && cut < 0 && ti >= 0) {
-      const double* fr = a.ftab + (int64_t)ti * MAXK;
-      for (int i = 0; i < K; ++i) row[i] = fr[i];
+      for (int i = 0; i < K; ++i) row[i] = a.ftab[(int64_t)i * TAB_N + ti];
       return w;
     }
     if (kind == 1 && a.eb_bc && a.eb_bc[cut] != 0) {
@@ -595,15 +566,9 @@ __device__ __forceinline__ T column_sums(const T* P, int c0, int mm, int lane, i
 
 // sign and zero tests on the bit patterns (integer pipe)
 __device__ __forceinline__ bool bits_nonzero(double v) { return __double_as_longlong(v) != 0; }
-__device__ __forceinline__ bool bits_nonzero(float v) { return __float_as_int(v) != 0; }
 __device__ __forceinline__ bool bits_positive(double v) { return __double_as_longlong(v) > 0; }
-__device__ __forceinline__ bool bits_positive(float v) { return __float_as_int(v) > 0; }
 
 constexpr uint32_t PAIR_WAIT_LIMIT = 1000000u;
-constexpr int LS_MAX_CORR = 8;             // corrections of the FP32-factorisation path
-constexpr double LS_CORR_TOL = 1e-14;      // converged: the last correction moved t by at most this (2-norm, relative)
-constexpr double LS_CORR_FLOOR = 1e-11;    // ... or by at most this and less than half the one before (rounding floor)
-constexpr float LS_F32_MIN_DIAG = 2e-5f;   // FP32 factor with min |R_kk| below this times the largest: FP64 path
 
 // Barrier of the two warps of one system: every lane arrives on the system's mbarrier (64 arrivals
 // complete a phase; arrive releases, the wait acquires), then waits for the phase.  The wait is
@@ -638,34 +603,26 @@ __device__ __forceinline__ bool pair_sync(unsigned long long* bar, uint32_t& pha
 // column k+1 (the next vector, updated by its owner and read by the others after a group barrier)
 // and its scalars (posted by the owner with a sequence flag and read at the start of the next step).
 //
-// QT = double: the FP64 factorisation, the rank test |R_kk| <= 1e-12 max |R_jj| and one correction of
-// the semi-normal equations (t = B z, z = R^-1 R^-T F; t += B R^-1 R^-T (F - B^T t)).
-// QT = float: the rows are built in FP64 (kept for the corrections) and factorised in FP32; the FP32
-// factor preconditions FP64 corrections of the semi-normal equations, repeated until a correction moves
-// t by at most LS_CORR_TOL, or stops shrinking at the rounding floor (B R^-1 has singular values within
-// 1 +- cond(B) eps_32 of one, so each correction gains about that factor; the corrections end at the
-// same rounding floor as the FP64 path).  A
-// system whose FP32 factor is too ill-conditioned for that, or whose corrections do not settle within
-// LS_MAX_CORR, gets status 3 and is solved again by the FP64 kernel (which also makes the rank test).
+// The FP64 path: EB_LS_FP64, and the systems the mixed path (eb_lsq.cu) leaves.  FP64 factorisation, the rank
+// test |R_kk| <= 1e-12 max |R_jj| and one correction of the semi-normal equations (t = B z, z = R^-1 R^-T F;
+// t += B R^-1 R^-T (F - B^T t)).
 //
 // BATCH: the systems of several geometries (same dimension and order) in one launch; the work counter,
 // the total system count, the scratch and the error word come from a0, each system's geometry data
 // from batch[g] with g found from the prefix sums of the systems per geometry (slot_base).
-template <bool BATCH, typename QT>
-__global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
+template <bool BATCH>
+__global__ void __launch_bounds__(LS_SYS * LS_NW * 32, 1)
     k_lsq(const __grid_constant__ LsArgs a0, const __grid_constant__ Tables T, const LsArgs* __restrict__ batch,
           const int64_t* __restrict__ slot_base, int n_geom) {
-  constexpr bool F32 = sizeof(QT) == 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sys = warp / LS_NW, h = warp % LS_NW;
-  LsSysSmem<QT>& S = reinterpret_cast<LsSysSmem<QT>*>(smem_raw)[sys];
+  LsSysSmem& S = reinterpret_cast<LsSysSmem*>(smem_raw)[sys];
   const int K = T.K;
-  const int gs = blockIdx.x * ls_sys<QT>() + sys;
+  const int gs = blockIdx.x * LS_SYS + sys;
   double* scr = a0.scratch + (int64_t)gs * LS_SCRATCH;  // column-major: scr[k * MAXROWS + i]
   double* scr_w = scr + (int64_t)MAXROWS * MAXK;
   double* scr_t = scr_w + MAXROWS;
-  double* stage = scr_t + MAXROWS;  // FP64 rows of the chunk (FP32 factorisation), row stride KST
   double* F = S.vec;
   double* y = S.vec + MAXK;
   double* z = S.vec + 2 * MAXK;
@@ -719,20 +676,15 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
       x0s[dface] = -0.5;
     }
     int bad = 0;
-    for (int i = lane + 32 * h; i < K * K; i += 32 * LS_NW) S.R[i] = (QT)0;
+    for (int i = lane + 32 * h; i < K * K; i += 32 * LS_NW) S.R[i] = 0.0;
     // ---- row-streamed Householder QR of B = W A: R accumulates the triangular factor
     for (int c0 = 0; c0 < n; c0 += CH) {
       // rows of the chunk (warp h builds the row slots r with r % LS_NW == h): table rows directly,
-      // shifted rows queued (one ballot mask per row slot) and shifted with every lane busy.  FP64
-      // factorisation: built in the chunk buffer; FP32: built in the FP64 staging rows, then rounded
-      // into the chunk buffer
+      // shifted rows queued (one ballot mask per row slot) and shifted with every lane busy
       constexpr int NSLOT = (RPL + LS_NW - 1) / LS_NW;
       unsigned pend[NSLOT];
       int npend = 0;
-      auto row_at = [&](int li) -> double* {
-        if constexpr (F32) return stage + li * KST;
-        else return reinterpret_cast<double*>(S.C) + li * KST;
-      };
+      auto row_at = [&](int li) -> double* { return S.C + li * KST; };
 #pragma unroll
       for (int rr = 0; rr < NSLOT; ++rr) {
         const int r = h + LS_NW * rr;
@@ -772,13 +724,7 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
         const int li = lane + 32 * r, i = c0 + li;
         const double* src = row_at(li);
         if (i < n) {
-          for (int k = 0; k < K; ++k) {
-            const double v = src[k];
-            scr[(int64_t)k * MAXROWS + i] = v;
-            if constexpr (F32) S.C[li * KST + k] = (QT)v;
-          }
-        } else if constexpr (F32) {
-          for (int k = 0; k < K; ++k) S.C[li * KST + k] = (QT)0;
+          for (int k = 0; k < K; ++k) scr[(int64_t)k * MAXROWS + i] = src[k];
         }
       }
       PAIR_SYNC();  // the chunk's rows are complete
@@ -787,14 +733,14 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
       // Householder steps k = 0..K-1 on [R; C].  The update of step k and the partial dot products of
       // step k+1 share one pass: column k+1 is updated first by its owner (it is step k+1's Householder
       // vector), then each warp loads, updates, stores and dots its own later columns.
-      QT ck[RPL];
+      double ck[RPL];
 #pragma unroll
-      for (int r = 0; r < RPL; ++r) ck[r] = r < nr ? S.C[(lane + 32 * r) * KST] : (QT)0;
-      QT* Pl = S.P + lane * KST;
+      for (int r = 0; r < RPL; ++r) ck[r] = r < nr ? S.C[(lane + 32 * r) * KST] : 0.0;
+      double* Pl = S.P + lane * KST;
       {  // partial dots of column 0 with the own columns j >= 1
-        const QT* Cl = S.C + lane * KST;
+        const double* Cl = S.C + lane * KST;
         for (int j = 1 + (h + LS_NW - 1) % LS_NW; j < K; j += LS_NW) {
-          QT pp = 0;
+          double pp = 0;
 #pragma unroll
           for (int r = 0; r < RPL; ++r)
             if (r < nr) pp = fma(ck[r], Cl[32 * r * KST + j], pp);
@@ -802,21 +748,21 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
         }
       }
       // Householder scalars of step k from its vector (chunk part c, R part alpha = R_kk)
-      auto hscalars = [&](const QT* c, int k, QT* out) {
-        QT ss = c[0] * c[0];
+      auto hscalars = [&](const double* c, int k, double* out) {
+        double ss = c[0] * c[0];
 #pragma unroll
         for (int r = 1; r < RPL; ++r) ss = fma(c[r], c[r], ss);
         ss = warp_sum(ss);
         // a zero chunk column needs no reflection
         const bool refl = bits_nonzero(ss);
-        const QT alpha = S.R[k * K + k];
-        const QT sigma = refl ? sqrt(fma(alpha, alpha, ss)) : (QT)0;
+        const double alpha = S.R[k * K + k];
+        const double sigma = refl ? sqrt(fma(alpha, alpha, ss)) : 0.0;
         out[0] = bits_positive(alpha) ? -sigma : sigma;  // beta
         out[1] = alpha - out[0];                          // v0
-        out[2] = refl ? (QT)-1 / (out[0] * out[1]) : (QT)0;  // gamma
-        out[3] = refl ? (QT)1 : (QT)0;
+        out[2] = refl ? -1.0 / (out[0] * out[1]) : 0.0;  // gamma
+        out[3] = refl ? 1.0 : 0.0;
       };
-      QT hk[4], hnext[4] = {0, 0, 0, 0};
+      double hk[4], hnext[4] = {0, 0, 0, 0};
       hscalars(ck, 0, hk);  // step 0: both warps (the vector is column 0)
       for (int k = 0; k < K; ++k, ++stepno) {
         if (k > 0 && h != k % LS_NW) {
@@ -837,7 +783,7 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
 #pragma unroll
           for (int q = 0; q < 4; ++q) hk[q] = hnext[q];  // this warp computed them in step k-1
         }
-        const QT beta = hk[0], v0 = hk[1], gamma = hk[2];
+        const double beta = hk[0], v0 = hk[1], gamma = hk[2];
         const bool refl = bits_nonzero(hk[3]);  // 1 or 0
         __syncwarp();  // P holds the partial dots of column k with the own later columns
         const int jf = k + 1 + (h + LS_NW - (k + 1) % LS_NW) % LS_NW;  // first own column after k
@@ -845,24 +791,24 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
         for (int c1 = 0; c1 < mown; c1 += 32) {
           const int mm = mown - c1 < 32 ? mown - c1 : 32;
           int col;
-          const QT sum = column_sums<LS_NW>(S.P, jf + LS_NW * c1, mm, lane, &col);
+          const double sum = column_sums<LS_NW>(S.P, jf + LS_NW * c1, mm, lane, &col);
           if (col >= 0) {
             const int j = jf + LS_NW * (c1 + col);
-            const QT rkj = S.R[k * K + j];
-            const QT t = gamma * fma(v0, rkj, sum);
+            const double rkj = S.R[k * K + j];
+            const double t = gamma * fma(v0, rkj, sum);
             if (refl) S.R[k * K + j] = fma(-t, v0, rkj);
-            tau[j] = (double)t;
+            tau[j] = t;
           }
         }
         __syncwarp();
         if (k + 1 < K) {
           const int owner = (k + 1) % LS_NW;
-          QT ck1[RPL];
+          double ck1[RPL];
           if (h == owner) {  // column k+1: update, keep as the next Householder vector
-            const QT t1 = (QT)tau[k + 1];
+            const double t1 = tau[k + 1];
 #pragma unroll
             for (int r = 0; r < RPL; ++r) {
-              QT* c = S.C + (lane + 32 * r) * KST + k + 1;
+              double* c = S.C + (lane + 32 * r) * KST + k + 1;
               ck1[r] = 0;
               if (r < nr) {
                 ck1[r] = fma(-t1, ck[r], *c);
@@ -873,10 +819,10 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
           PAIR_SYNC();
           if (h != owner) {
 #pragma unroll
-            for (int r = 0; r < RPL; ++r) ck1[r] = r < nr ? S.C[(lane + 32 * r) * KST + k + 1] : (QT)0;
+            for (int r = 0; r < RPL; ++r) ck1[r] = r < nr ? S.C[(lane + 32 * r) * KST + k + 1] : 0.0;
           } else {
             // step k+1's scalars, off the other warp's path: it picks them up at the start of step k+1
-            QT hn[4];
+            double hn[4];
             hscalars(ck1, k + 1, hn);  // R_{k+1,k+1} is not touched by step k
             if (lane == 0) {
 #pragma unroll
@@ -891,14 +837,14 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
           constexpr int W = LS_NW;
           int j = k + 2 + (h + W - (k + 2) % W) % W;
           for (; j + 3 * W < K; j += 4 * W) {
-            const QT t0 = (QT)tau[j], tt1 = (QT)tau[j + W], t2 = (QT)tau[j + 2 * W], t3 = (QT)tau[j + 3 * W];
-            QT q0 = 0, q1 = 0, q2 = 0, q3 = 0;
+            const double t0 = tau[j], tt1 = tau[j + W], t2 = tau[j + 2 * W], t3 = tau[j + 3 * W];
+            double q0 = 0, q1 = 0, q2 = 0, q3 = 0;
 #pragma unroll
             for (int r = 0; r < RPL; ++r) {
               if (r < nr) {
-                QT* c = S.C + (lane + 32 * r) * KST + j;
-                const QT e0 = fma(-t0, ck[r], c[0]), e1 = fma(-tt1, ck[r], c[W]);
-                const QT e2 = fma(-t2, ck[r], c[2 * W]), e3 = fma(-t3, ck[r], c[3 * W]);
+                double* c = S.C + (lane + 32 * r) * KST + j;
+                const double e0 = fma(-t0, ck[r], c[0]), e1 = fma(-tt1, ck[r], c[W]);
+                const double e2 = fma(-t2, ck[r], c[2 * W]), e3 = fma(-t3, ck[r], c[3 * W]);
                 c[0] = e0;
                 c[W] = e1;
                 c[2 * W] = e2;
@@ -915,13 +861,13 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
             Pl[j + 3 * W] = q3;
           }
           for (; j < K; j += W) {
-            const QT t0 = (QT)tau[j];
-            QT q0 = 0;
+            const double t0 = tau[j];
+            double q0 = 0;
 #pragma unroll
             for (int r = 0; r < RPL; ++r) {
               if (r < nr) {
-                QT* c = S.C + (lane + 32 * r) * KST + j;
-                const QT e0 = fma(-t0, ck[r], c[0]);
+                double* c = S.C + (lane + 32 * r) * KST + j;
+                const double e0 = fma(-t0, ck[r], c[0]);
                 c[0] = e0;
                 q0 = fma(ck1[r], e0, q0);
               }
@@ -936,27 +882,16 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
       }
       PAIR_SYNC();  // both warps are done with the chunk and with R
     }
-    // ---- rank check (FP64: |R_kk| <= 1e-12 max |R_jj| counts as rank deficient; FP32: a factor that
-    // ill-conditioned leaves the system to the FP64 kernel)
-    const int anyb = __any_sync(0xffffffffu, bad);
-    if (lane == 0) S.bad[h] = anyb;
-    PAIR_SYNC();
-    {
-      int any = 0;
-      for (int q = 0; q < LS_NW; ++q) any |= S.bad[q];
-      bad = any ? 2 : 0;
-    }
+    // ---- rank check: |R_kk| <= 1e-12 max |R_jj| counts as rank deficient
     double dmax = 0.0, dmin = INFINITY;
     for (int k = 0; k < K; ++k) {
-      double v = fabs((double)S.R[k * K + k]);
+      double v = fabs(S.R[k * K + k]);
       dmax = fmax(dmax, v);
       dmin = fmin(dmin, v);
     }
-    if (!bad && !(dmin > (F32 ? (double)LS_F32_MIN_DIAG : 1e-12) * dmax)) bad = F32 ? 3 : 1;
-    if (bad) {
-      if (h == 0 && lane == 0) a.status[s] = bad;
-      if (bad != 3)
-        for (int i = lane + 32 * h; i < n; i += 32 * LS_NW) a.row_val[p0 + i] = 0.0;
+    if (!(dmin > 1e-12 * dmax)) {
+      if (h == 0 && lane == 0) a.status[s] = 1;
+      for (int i = lane + 32 * h; i < n; i += 32 * LS_NW) a.row_val[p0 + i] = 0.0;
       PAIR_SYNC();
       continue;
     }
@@ -967,7 +902,7 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
       for (int k = 0; k < K; ++k) {  // R^T y = rhs (forward)
         double yk = y[k] * rinv[k];
         __syncwarp();
-        for (int j = k + 1 + lane; j < K; j += 32) y[j] = fma(-(double)S.R[k * K + j], yk, y[j]);
+        for (int j = k + 1 + lane; j < K; j += 32) y[j] = fma(-S.R[k * K + j], yk, y[j]);
         if (lane == 0) y[k] = yk;
         __syncwarp();
       }
@@ -976,13 +911,13 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
       for (int k = K - 1; k >= 0; --k) {  // R z = y (backward)
         double zk = outz[k] * rinv[k];
         __syncwarp();
-        for (int j = lane; j < k; j += 32) outz[j] = fma(-(double)S.R[j * K + k], zk, outz[j]);
+        for (int j = lane; j < k; j += 32) outz[j] = fma(-S.R[j * K + k], zk, outz[j]);
         if (lane == 0) outz[k] = zk;
         __syncwarp();
       }
     };
     if (h == 0) {
-      for (int k = lane; k < K; k += 32) rinv[k] = 1.0 / (double)S.R[k * K + k];
+      for (int k = lane; k < K; k += 32) rinv[k] = 1.0 / S.R[k * K + k];
       // ---- F_hat (Sec. 2.2.1): grid face: p_d m_f^{p-e_d}; EB face: sum_d p_d m_{d,f}^{p-e_d}
       for (int i = lane; i < K; i += 32) {
         double f = 0.0;
@@ -1007,106 +942,47 @@ __global__ void __launch_bounds__(ls_sys<QT>() * LS_NW * 32, 1)
       solve_rtr(F, z);
     }
     PAIR_SYNC();
-    // ---- corrected semi-normal equations: t = B z, then corrections t += B R^-1 R^-T (F - B^T t).
-    // FP64 factorisation: one correction, B^T t from per-lane partials over the rows (warps h > 0 in the
-    // free chunk buffer) and column sums.  FP32: lanes own columns and each warp sums half of the rows
-    // (the chunk buffer is too small for the partials in FP64)
+    // ---- corrected semi-normal equations: t = B z, then one correction t += B R^-1 R^-T (F - B^T t), B^T t
+    // from per-lane partials over the rows (warps h > 0 in the free chunk buffer) and column sums
     for (int i = lane + 32 * h; i < n; i += 32 * LS_NW) {
       double t1 = 0.0;
       for (int k = 0; k < K; ++k) t1 = fma(scr[(int64_t)k * MAXROWS + i], z[k], t1);
       scr_t[i] = t1;
     }
-    double* z2 = reinterpret_cast<double*>(S.C) + (CH * KST * sizeof(QT)) / 8 - 2 * MAXK;  // the chunk buffer's tail
-    bool settled = false;
-    double prev_sd = INFINITY;  // the previous correction's squared norm
-    int ncorr = 0;
-    for (int corr = 0; corr < (F32 ? LS_MAX_CORR : 1) && !settled; ++corr) {
-      ++ncorr;
-      if constexpr (F32) {
-        PAIR_SYNC();  // t is complete
-        const int i0 = h * ((n + 1) >> 1), i1 = h ? n : (n + 1) >> 1;
-        double s0 = 0.0, s1 = 0.0;
-        const double* c0p = scr + (int64_t)lane * MAXROWS;
-        const double* c1p = scr + (int64_t)(lane + 32) * MAXROWS;
-        for (int i = i0; i < i1; ++i) {
-          const double t1 = scr_t[i];
-          if (lane < K) s0 = fma(c0p[i], t1, s0);
-          if (lane + 32 < K) s1 = fma(c1p[i], t1, s1);
-        }
-        if (lane < K) S.xch[h * MAXK + lane] = s0;
-        if (lane + 32 < K) S.xch[h * MAXK + lane + 32] = s1;
-      } else {
-        double* Pw = h == 0 ? reinterpret_cast<double*>(S.P) : reinterpret_cast<double*>(S.C) + (h - 1) * 32 * KST;
-        for (int k = 0; k < K; ++k) Pw[lane * KST + k] = 0.0;
-        for (int i = lane + 32 * h; i < n; i += 32 * LS_NW) {
-          const double t1 = scr_t[i];
-          for (int k = 0; k < K; ++k) Pw[lane * KST + k] = fma(scr[(int64_t)k * MAXROWS + i], t1, Pw[lane * KST + k]);
-        }
-        __syncwarp();
-        for (int c1 = 0; c1 < K; c1 += 32) {
-          int mm = K - c1 < 32 ? K - c1 : 32;
-          int col;
-          double sum = column_sums<1>(Pw, c1, mm, lane, &col);
-          if (col >= 0) S.xch[h * MAXK + c1 + col] = sum;
-        }
+    double* z2 = S.C + CH * KST - 2 * MAXK;  // the chunk buffer's tail
+    double* Pw = h == 0 ? S.P : S.C + (h - 1) * 32 * KST;
+    for (int k = 0; k < K; ++k) Pw[lane * KST + k] = 0.0;
+    for (int i = lane + 32 * h; i < n; i += 32 * LS_NW) {
+      const double t1 = scr_t[i];
+      for (int k = 0; k < K; ++k) Pw[lane * KST + k] = fma(scr[(int64_t)k * MAXROWS + i], t1, Pw[lane * KST + k]);
+    }
+    __syncwarp();
+    for (int c1 = 0; c1 < K; c1 += 32) {
+      int mm = K - c1 < 32 ? K - c1 : 32;
+      int col;
+      double sum = column_sums<1>(Pw, c1, mm, lane, &col);
+      if (col >= 0) S.xch[h * MAXK + c1 + col] = sum;
+    }
+    PAIR_SYNC();
+    if (h == 0) {
+      for (int c = lane; c < K; c += 32) {
+        double sx = 0.0;
+        for (int q = 0; q < LS_NW; ++q) sx += S.xch[q * MAXK + c];
+        tau[c] = F[c] - sx;
       }
-      PAIR_SYNC();
-      if (h == 0) {
-        for (int c = lane; c < K; c += 32) {
-          double sx = 0.0;
-          for (int q = 0; q < LS_NW; ++q) sx += S.xch[q * MAXK + c];
-          tau[c] = F[c] - sx;
-        }
-        __syncwarp();
-        solve_rtr(tau, z2);
-      }
-      PAIR_SYNC();
-      if constexpr (F32) {
-        double dd = 0.0, tt = 0.0;  // the correction's and the result's squared norms (this warp's rows)
-        for (int i = lane + 32 * h; i < n; i += 32 * LS_NW) {
-          double dt = 0.0;
-          for (int k = 0; k < K; ++k) dt = fma(scr[(int64_t)k * MAXROWS + i], z2[k], dt);
-          const double t = scr_t[i] + dt;
-          scr_t[i] = t;
-          dd = fma(dt, dt, dd);
-          tt = fma(t, t, tt);
-        }
-        dd = warp_sum(dd);
-        tt = warp_sum(tt);
-        __syncwarp();
-        if (lane == 0) {
-          S.xch[h * MAXK] = dd;
-          S.xch[h * MAXK + 1] = tt;
-        }
-        PAIR_SYNC();
-        double sd = 0.0, st = 0.0;
-        for (int q = 0; q < LS_NW; ++q) {
-          sd += S.xch[q * MAXK];
-          st += S.xch[q * MAXK + 1];
-        }
-        settled = sd <= LS_CORR_TOL * LS_CORR_TOL * st ||
-                  (sd <= LS_CORR_FLOOR * LS_CORR_FLOOR * st && sd > 0.25 * prev_sd);
-        prev_sd = sd;
-      } else {
-        for (int i = lane + 32 * h; i < n; i += 32 * LS_NW) {
-          double t = scr_t[i];
-          for (int k = 0; k < K; ++k) t = fma(scr[(int64_t)k * MAXROWS + i], z2[k], t);
-          scr_t[i] = t;
-        }
-        settled = true;
-      }
+      __syncwarp();
+      solve_rtr(tau, z2);
+    }
+    PAIR_SYNC();
+    for (int i = lane + 32 * h; i < n; i += 32 * LS_NW) {
+      double t = scr_t[i];
+      for (int k = 0; k < K; ++k) t = fma(scr[(int64_t)k * MAXROWS + i], z2[k], t);
+      scr_t[i] = t;
     }
     if (h == 0 && lane == 0 && a0.flops) {  // executed flops of this system (the row construction not counted)
       const double nn = n, kk = K;
       const double fact = 2.0 * nn * kk * kk - 2.0 / 3.0 * kk * kk * kk;  // Householder QR of n x K
-      const double semi = 2.0 * nn * kk + 2.0 * kk * kk + ncorr * (4.0 * nn * kk + 2.0 * kk * kk);
-      atomicAdd(a0.flops + 0, F32 ? semi : fact + semi);
-      if (F32) atomicAdd(a0.flops + 1, fact);
-    }
-    if (!settled) {  // FP32 factor: the corrections did not settle; the FP64 kernel takes the system
-      if (h == 0 && lane == 0) a.status[s] = 3;
-      PAIR_SYNC();
-      continue;
+      atomicAdd(a0.flops + 0, fact + 2.0 * nn * kk + 2.0 * kk * kk + 4.0 * nn * kk + 2.0 * kk * kk);
     }
     for (int i = lane + 32 * h; i < n; i += 32 * LS_NW) a.row_val[p0 + i] = scr_w[i] * scr_t[i];  // s_hat = W t
     if (h == 0 && lane == 0) a.status[s] = a0.slot_list ? 4 : 0;  // 4: solved by the FP64 pass after the FP32 one
@@ -1253,16 +1129,10 @@ __global__ void k_assemble_b(AsmArgs a, const int32_t* __restrict__ cells, int64
 
 namespace eb {
 
-size_t lsq_smem(bool fp32) {
-  return fp32 ? (size_t)LS_SYS_F * sizeof(LsSysSmem<float>) : (size_t)LS_SYS * sizeof(LsSysSmem<double>);
-}
-
 cudaError_t lsq_prepare() {
-  const int sd = (int)lsq_smem(false), sf = (int)lsq_smem(true);
-  cudaError_t e = cudaFuncSetAttribute(k_lsq<false, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, sd);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lsq<true, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, sd);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lsq<false, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, sf);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lsq<true, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, sf);
+  const int sd = (int)(LS_SYS * sizeof(LsSysSmem));
+  cudaError_t e = cudaFuncSetAttribute(k_lsq<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sd);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lsq<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sd);
   return e;
 }
 
@@ -1595,18 +1465,12 @@ cudaError_t stencil_adjoint_launch(unsigned blocks, cudaStream_t s, const LsArgs
   return cudaGetLastError();
 }
 
-cudaError_t lsq_launch(bool fp32, unsigned blocks, cudaStream_t s, const LsArgs& a0, const Tables& T,
-                       const LsArgs* batch, const int64_t* slot_base, int n_geom) {
-  const size_t smem = lsq_smem(fp32);
-  if (fp32) {
-    constexpr unsigned nt = LS_SYS_F * LS_NW * 32;
-    if (batch) k_lsq<true, float><<<blocks, nt, smem, s>>>(a0, T, batch, slot_base, n_geom);
-    else k_lsq<false, float><<<blocks, nt, smem, s>>>(a0, T, nullptr, nullptr, 1);
-  } else {
-    constexpr unsigned nt = LS_SYS * LS_NW * 32;
-    if (batch) k_lsq<true, double><<<blocks, nt, smem, s>>>(a0, T, batch, slot_base, n_geom);
-    else k_lsq<false, double><<<blocks, nt, smem, s>>>(a0, T, nullptr, nullptr, 1);
-  }
+cudaError_t lsq_launch(unsigned blocks, cudaStream_t s, const LsArgs& a0, const Tables& T, const LsArgs* batch,
+                       const int64_t* slot_base, int n_geom) {
+  const size_t smem = LS_SYS * sizeof(LsSysSmem);
+  constexpr unsigned nt = LS_SYS * LS_NW * 32;
+  if (batch) k_lsq<true><<<blocks, nt, smem, s>>>(a0, T, batch, slot_base, n_geom);
+  else k_lsq<false><<<blocks, nt, smem, s>>>(a0, T, nullptr, nullptr, 1);
   return cudaGetLastError();
 }
 

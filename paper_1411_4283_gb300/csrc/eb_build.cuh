@@ -24,57 +24,54 @@ struct GatherArgs {
   const int64_t* row_ptr;    // null in the counting pass
   uint32_t* row_desc;
   int64_t* count;            // [n_slots] counting pass output
-  int32_t* too_many;         // capacity flag
+  int32_t* max_rows;         // counting pass: most rows of a slot
 };
 
-// LS kernel shape (compile-time; EB_LS_SYS / EB_LS_SYS_F / EB_LS_RPL override it for tuning builds)
+// LS kernel shapes (compile-time; EB_LS_W / EB_LS_CTAS / EB_LS_SYS / EB_LS_RPL override them for tuning builds)
+#ifndef EB_LS_W
+#define EB_LS_W 4
+#endif
+#ifndef EB_LS_CTAS
+#define EB_LS_CTAS 2
+#endif
 #ifndef EB_LS_SYS
 #define EB_LS_SYS 4
-#endif
-#ifndef EB_LS_SYS_F
-#define EB_LS_SYS_F 6
 #endif
 #ifndef EB_LS_RPL
 #define EB_LS_RPL 4
 #endif
-constexpr int LS_SYS = EB_LS_SYS;      // systems in flight per CTA, FP64 factorisation (shared memory bound)
-constexpr int LS_SYS_F = EB_LS_SYS_F;  // systems in flight per CTA, FP32 factorisation
-constexpr int LS_NW = 2;               // warps per system (each owns the columns j with j % LS_NW == its rank)
-constexpr int RPL = EB_LS_RPL;  // rows per lane per chunk
-constexpr int CH = 32 * RPL;  // rows per chunk
-constexpr int KST = MAXK;     // row stride in shared memory (odd: conflict-free 32- and 64-bit access)
-template <typename QT>
-__host__ __device__ constexpr int ls_sys() {
-  return sizeof(QT) == 8 ? LS_SYS : LS_SYS_F;
-}
+constexpr int LS_SYS = EB_LS_SYS;  // systems in flight per CTA, FP64 factorisation (shared memory bound)
+constexpr int LS_NW = 2;           // warps per system (each owns the columns j with j % LS_NW == its rank)
+constexpr int RPL = EB_LS_RPL;     // rows per lane per chunk
+constexpr int CH = 32 * RPL;       // rows per chunk
+constexpr int KST = MAXK;          // row stride in shared memory (odd: conflict-free 64-bit access)
 
-// Per-system shared memory; QT is the precision of the factorisation (the corrected semi-normal
-// equations run in FP64 either way)
-template <typename QT>
+// Per-system shared memory of the FP64 factorisation
 struct __align__(16) LsSysSmem {
-  QT R[MAXK * MAXK + 1];     // triangular factor, row-major (one pad entry keeps C 8-byte aligned)
-  QT C[CH * KST];            // current chunk of weighted rows
-  QT P[32 * KST];            // partial dot products, column j in P[lane][j] (each column owned by one warp)
-  double vec[5 * MAXK];      // F, y, z, tau, 1/R_kk
-  double xch[LS_NW * MAXK];  // the warps' partial sums (corrected semi-normal equations)
-  QT hs[2][4];               // Householder scalars (beta, v0, gamma, reflect) of step k in hs[k % 2]
-  unsigned long long bar;    // barrier of the system's warps (mbarrier, 32 * LS_NW arrivals per phase)
-  int32_t slot;              // system being solved
-  int32_t bad[LS_NW];        // per-warp row flags
-  int32_t hs_seq[2];         // step number whose scalars hs[k % 2] holds (posted after the values)
-  int32_t done;              // corrections converged (FP32 factorisation)
+  double R[MAXK * MAXK + 1];  // triangular factor, row-major
+  double C[CH * KST];         // current chunk of weighted rows
+  double P[32 * KST];         // partial dot products, column j in P[lane][j] (each column owned by one warp)
+  double vec[5 * MAXK];       // F, y, z, tau, 1/R_kk
+  double xch[LS_NW * MAXK];   // the warps' partial sums (corrected semi-normal equations)
+  double hs[2][4];            // Householder scalars (beta, v0, gamma, reflect) of step k in hs[k % 2]
+  unsigned long long bar;     // barrier of the system's warps (mbarrier, 32 * LS_NW arrivals per phase)
+  int32_t slot;               // system being solved
+  int32_t hs_seq[2];          // step number whose scalars hs[k % 2] holds (posted after the values)
 };
-static_assert(sizeof(LsSysSmem<double>) % 16 == 0 && sizeof(LsSysSmem<float>) % 16 == 0,
-              "per-system blocks stay 16-byte aligned");
-static_assert(LS_SYS * sizeof(LsSysSmem<double>) <= 232448 && LS_SYS_F * sizeof(LsSysSmem<float>) <= 232448,
-              "the systems of a CTA fit in 227 KB of shared memory");
-// per-system global scratch (doubles): the rows column-major (MAXROWS x MAXK), the weights and t
-// (MAXROWS each), and the FP64 row staging of the FP32 factorisation (CH x KST)
-constexpr int64_t LS_SCRATCH = (int64_t)MAXROWS * (MAXK + 2) + (int64_t)CH * KST;
+static_assert(sizeof(LsSysSmem) % 16 == 0, "per-system blocks stay 16-byte aligned");
+static_assert(LS_SYS * sizeof(LsSysSmem) <= 232448, "the systems of a CTA fit in 227 KB of shared memory");
+// per-system global scratch (doubles) of the FP64 factorisation: the rows column-major (MAXROWS x MAXK),
+// the weights and t (MAXROWS each)
+constexpr int64_t LS_SCRATCH = (int64_t)MAXROWS * (MAXK + 2);
 
 // offsets in units of h/2 span [-11, 11] on each axis (volume, EB and wall rows)
 constexpr int TAB_S = 23;
 constexpr int TAB_N = TAB_S * TAB_S * TAB_S;
+// Place of the offset with indices x (0..TAB_S-1 each): even x first, then odd ones, so that the rows of
+// neighbouring cells (two half-cells apart) are next to each other
+__host__ __device__ inline int tab_place(const int* x) {
+  return (x[0] & 1) * ((TAB_S + 1) / 2) + (x[0] >> 1) + TAB_S * (x[1] + TAB_S * x[2]);
+}
 
 struct LsArgs {
   Dims dm;
@@ -96,11 +93,15 @@ struct LsArgs {
   const int32_t* slot_list;  // [n_slots] systems to solve (null: 0 .. n_slots-1)
   int32_t* next;       // work counter
   int32_t* status;     // [n_slots]: 0 ok, 1 rank deficient, 2 unsupported row, 3 left to the FP64 path
-  double* scratch;     // per system in flight: LS_SCRATCH doubles
+  double* scratch;     // per system in flight: LS_SCRATCH doubles (FP64), see k_lsq_mixed (mixed)
   int32_t* err;        // set when a bounded wait between the two warps of a system gives up
-  double* flops;       // [2] executed flops, accumulated: FP64 (factorisation, corrections), FP32 (factorisation)
-  const double* ftab;  // [TAB_N][MAXK] weighted rows of full cells, by offset
-  const double* wtab;  // [TAB_N] weights, by offset
+  double* flops;       // [2] executed flops, accumulated: FP64, FP32
+  // weighted rows of full cells by offset (tab_place): entry k at [k * TAB_N + place], FP64 and as the sum of
+  // two FP32 numbers, and the weights [TAB_N]
+  const double* ftab;
+  const float* ftab_h;
+  const float* ftab_l;
+  const double* wtab;
 };
 
 struct AsmArgs {
@@ -153,17 +154,20 @@ constexpr int ADJ_WARPS = 4;
 constexpr int ADJ_SCRATCH = MAXK + 10;  // doubles per row of a warp's scratch
 cudaError_t stencil_adjoint_launch(unsigned blocks, cudaStream_t s, const LsArgs& a, const Tables& T,
                                    const AdjArgs& g);
-// k_lsq launchers (eb_build.cu): shared-memory attribute, then one launch over the systems of one
+// FP64 factorisation (k_lsq, eb_build.cu): shared-memory attribute, then one launch over the systems of one
 // geometry (batch == null) or of several (batch[g] per geometry, slot_base prefix sums of their systems)
-// fp32: the FP32-factorisation kernel (systems it cannot finish get status 3), else the FP64 one
 cudaError_t lsq_prepare();
-size_t lsq_smem(bool fp32);
-cudaError_t lsq_launch(bool fp32, unsigned blocks, cudaStream_t s, const LsArgs& a0, const Tables& T,
-                       const LsArgs* batch, const int64_t* slot_base, int n_geom);
+cudaError_t lsq_launch(unsigned blocks, cudaStream_t s, const LsArgs& a0, const Tables& T, const LsArgs* batch,
+                       const int64_t* slot_base, int n_geom);
+// Mixed path (k_lsq_mixed, eb_lsq.cu), systems of at most max_rows rows: its blocks and the scratch they need,
+// and the launch; the systems it cannot finish get status 3
+int64_t lsq_mixed_blocks(const Tables& T, int max_rows, int64_t systems, int nsm, int64_t* scratch_doubles);
+cudaError_t lsq_mixed_launch(int64_t blocks, int max_rows, cudaStream_t s, const LsArgs& a0, const Tables& T,
+                             const LsArgs* batch, const int64_t* slot_base, int n_geom);
 // the systems with status 3 (global numbers: + base) appended to list[*count]
 cudaError_t lsq_fallback_list(const int32_t* status, int64_t n, int64_t base, int32_t* list, int32_t* count,
                               cudaStream_t s);
-__global__ void k_full_rows(Dims dm, const Tables* T, double* ftab, double* wtab);
+__global__ void k_full_rows(Dims dm, const Tables* T, double* ftab, float* ftab_h, float* ftab_l, double* wtab);
 __global__ void k_assemble_rows(AsmArgs a, const int32_t* rep_cell, int64_t nrep, int64_t row0, int32_t* err);
 __global__ void k_assemble_b(AsmArgs a, const int32_t* cells, int64_t ncells, int64_t* cnt, const int64_t* bptr,
                              int64_t* bcol, double* bval, const int32_t* unused);

@@ -303,7 +303,12 @@ __global__ void k_cell_kind(Dims dm, const uint8_t* flag, const int32_t* fs0, co
       if (sl != tmpl_slot[d]) tmpl = false;
     }
   if (uniq) { kind[c] = 2; rowkey[c] = -2; is_unique[c] = 1; return; }
-  if (tmpl) { kind[c] = 1; rowkey[c] = 0; atomicMin((unsigned long long*)&row_rep[0], (unsigned long long)c); return; }
+  // a class's lowest cell; most cells share one class, and few of them are lower than the ones before
+  auto rep = [&](int key) {
+    if ((unsigned long long)c < *(volatile unsigned long long*)&row_rep[key])
+      atomicMin((unsigned long long*)&row_rep[key], (unsigned long long)c);
+  };
+  if (tmpl) { kind[c] = 1; rowkey[c] = 0; rep(0); return; }
   kind[c] = 2;
   int M = dm.R + 3, key = 0;
   for (int k = dm.dim - 1; k >= 0; --k) {
@@ -314,7 +319,7 @@ __global__ void k_cell_kind(Dims dm, const uint8_t* flag, const int32_t* fs0, co
   }
   key += 1;  // 0 is the template
   rowkey[c] = key;
-  atomicMin((unsigned long long*)&row_rep[key], (unsigned long long)c);
+  rep(key);
 }
 
 __global__ void k_irr_list(int64_t ncell, const uint8_t* kind, const int64_t* pos, const int32_t* rowkey,
@@ -592,7 +597,7 @@ struct BuildCtx {
   cudaStream_t s = nullptr;
   eb_params P;
   int R = 0, D = 0, nsm = 0, max_rows = 0;
-  int64_t N = 0, n_slots = 0, n_unique = 0;
+  int64_t N = 0, n_slots = 0, n_unique = 0, nnz = 0;  // nnz: rows of all systems
   Tables T;
   Tables* dT = nullptr;
   Tmp tmp;
@@ -1126,8 +1131,8 @@ static eb_status build_pre(BuildCtx& c) {
   ga.count = counts;
   ga.max_rows = max_rows;
   ga.row_ptr = nullptr;
-  k_gather<<<nblk(n_slots, 128), 128, 0, s>>>(ga, n_slots, st->cut_cell); eb::count_launch();
-  EB_CUDA(cudaGetLastError());
+  EB_CUDA(gather_launch(ga, n_slots, st->cut_cell, s));
+  eb::count_launch();
   EB_TRY(dalloc(st, &st->row_ptr, n_slots + 1));
   int64_t nnz = 0;
   EB_CUDA(cudaMemsetAsync(counts + n_slots, 0, 8, s));
@@ -1135,12 +1140,13 @@ static eb_status build_pre(BuildCtx& c) {
   EB_CUDA(cudaMemcpyAsync(&c.max_rows, max_rows, 4, cudaMemcpyDeviceToHost, s));
   EB_CUDA(cudaStreamSynchronize(s));
   if (c.max_rows > MAXROWS) { set_error("a face has more LS rows than the kernel supports"); return EB_ERR_CAPACITY; }
+  c.nnz = nnz;
   EB_TRY(dalloc(st, &st->row_desc, nnz));
   EB_TRY(dalloc(st, &st->row_val, nnz));
   ga.row_ptr = st->row_ptr;
   ga.row_desc = st->row_desc;
-  k_gather<<<nblk(n_slots, 128), 128, 0, s>>>(ga, n_slots, st->cut_cell); eb::count_launch();
-  EB_CUDA(cudaGetLastError());
+  EB_CUDA(gather_launch(ga, n_slots, st->cut_cell, s));
+  eb::count_launch();
   // ---- 4. weighted least squares (FP64): inputs here, the launch in build_ls
   int dev = 0, nsm = 0;
   EB_CUDA(cudaGetDevice(&dev));
@@ -1308,21 +1314,30 @@ static eb_status build_post(BuildCtx& c) {
   double* invk = c.invk;
   const int M = R + 3;
   {
-    std::vector<int32_t> hs(n_slots);
-    EB_CUDA(cudaMemcpyAsync(hs.data(), status, n_slots * 4, cudaMemcpyDeviceToHost, s));
-    EB_CUDA(cudaStreamSynchronize(s));
-    int unbuilt = 0, nbad = 0;
-    int64_t nfp64 = 0;
-    for (int64_t i = 0; i < n_slots; ++i) {
-      if (hs[i] == 1) ++nbad;
-      if (hs[i] == 2) unbuilt = 1;  // a row flagged by the row builder
-      if (hs[i] == 4) ++nfp64;      // left by the FP32 factorisation, solved by the FP64 one
+    // counted on the device: face states and system statuses (4: left by the mixed path, solved in FP64)
+    unsigned long long* counts;
+    unsigned long long hc[5];
+    EB_TRY(tmp.get(&counts, 5));
+    EB_CUDA(cudaMemsetAsync(counts, 0, sizeof(hc), s));
+    for (int d = 0; d < D; ++d) {
+      EB_CUDA(count_faces(st->face_slot[d], dm.nface[d], n_unique, counts, s));
+      eb::count_launch();
     }
-    info->n_ls_fp64 = c.P.ls_precision == EB_LS_FP64 ? n_slots : nfp64;
+    EB_CUDA(count_status(status, n_slots, counts, s));
+    eb::count_launch();
+    EB_CUDA(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
+    EB_CUDA(cudaStreamSynchronize(s));
+    info->n_flux_faces = (int64_t)hc[0] + nc;
+    info->n_class_faces = (int64_t)hc[1];
+    info->n_ls_fp64 = c.P.ls_precision == EB_LS_FP64 ? n_slots : (int64_t)hc[4];
     info->ls_fp64_flops = c.ls_flops[0];
     info->ls_fp32_flops = c.ls_flops[1];
+    const bool unbuilt = hc[3] > 0;  // a row flagged by the row builder
     if (unbuilt) { set_error("an LS row could not be built"); return EB_ERR_INVALID; }
-    if (nbad) {
+    if (hc[2] > 0) {
+      std::vector<int32_t> hs(n_slots);
+      EB_CUDA(cudaMemcpyAsync(hs.data(), status, n_slots * 4, cudaMemcpyDeviceToHost, s));
+      EB_CUDA(cudaStreamSynchronize(s));
       // every face whose system failed: a class slot stands for all the faces of its class, so the
       // faces are listed from the face -> slot maps (ascending global face id)
       for (int d = 0; d < D; ++d) {
@@ -1485,17 +1500,14 @@ static eb_status build_post(BuildCtx& c) {
     int64_t *bcnt, nbnz = 0;
     EB_TRY(tmp.get(&bcnt, st->n_irr + 1));
     EB_CUDA(cudaMemsetAsync(bcnt, 0, (st->n_irr + 1) * 8, s));
-    if (st->n_irr > 0)
-      k_assemble_b<<<nblk(st->n_irr, 128), 128, 0, s>>>(aa, st->irr_cell, st->n_irr, bcnt, nullptr, nullptr, nullptr,
-                                                        nullptr); eb::count_launch();
+    EB_CUDA(assemble_b_launch(aa, st->irr_cell, st->n_irr, bcnt, nullptr, nullptr, nullptr, s));
+    eb::count_launch();
     EB_TRY(dalloc(st, &st->b_ptr, st->n_irr + 1));
     EB_TRY(scan<int64_t>(bcnt, st->n_irr + 1, st->b_ptr, &nbnz, s, tmp));
     EB_TRY(dalloc(st, &st->b_col, nbnz));
     EB_TRY(dalloc(st, &st->b_val, nbnz));
-    if (st->n_irr > 0)
-      k_assemble_b<<<nblk(st->n_irr, 128), 128, 0, s>>>(aa, st->irr_cell, st->n_irr, nullptr, st->b_ptr, st->b_col,
-                                                        st->b_val, nullptr); eb::count_launch();
-    EB_CUDA(cudaGetLastError());
+    EB_CUDA(assemble_b_launch(aa, st->irr_cell, st->n_irr, nullptr, st->b_ptr, st->b_col, st->b_val, s));
+    eb::count_launch();
     int32_t h_aerr = 0;
     EB_CUDA(cudaMemcpyAsync(&h_aerr, aerr, 4, cudaMemcpyDeviceToHost, s));
     EB_CUDA(cudaStreamSynchronize(s));
@@ -1641,40 +1653,12 @@ static eb_status build_post(BuildCtx& c) {
   EB_CUDA(cudaStreamSynchronize(s));
   // ---- info
   info->n_unique_faces = n_unique;
-  info->n_class_faces = 0;
-  for (int d = 0; d < D; ++d) info->n_class_faces += dm.nface[d];  // refined below
-  {
-    int64_t n_open = 0, n_cls = 0;
-    for (int d = 0; d < D; ++d) {
-      std::vector<int32_t> hs(dm.nface[d]);
-      EB_CUDA(cudaMemcpyAsync(hs.data(), st->face_slot[d], dm.nface[d] * 4, cudaMemcpyDeviceToHost, s));
-      EB_CUDA(cudaStreamSynchronize(s));
-      for (int32_t v : hs) {
-        if (v >= 0) ++n_open;
-        if (v >= n_unique) ++n_cls;
-      }
-    }
-    info->n_flux_faces = n_open + nc;
-    info->n_class_faces = n_cls;
-  }
   info->n_classes = st->n_classes;
-  {
-    std::vector<int64_t> rp(n_slots + 1);
-    EB_CUDA(cudaMemcpyAsync(rp.data(), st->row_ptr, (n_slots + 1) * 8, cudaMemcpyDeviceToHost, s));
-    EB_CUDA(cudaStreamSynchronize(s));
-    int32_t mx = 0;
-    double fl = 0.0;
-    int K = T.K;
-    for (int64_t i = 0; i < n_slots; ++i) {
-      int64_t n = rp[i + 1] - rp[i];
-      mx = std::max<int32_t>(mx, (int32_t)n);
-      // the method's count per system: Householder QR of the n x K matrix, the triangular solve and the
-      // application of Q (2nK^2 - 2K^3/3 + 4nK + K^2)
-      fl += 2.0 * n * K * K - 2.0 / 3.0 * K * K * K + 4.0 * n * K + 1.0 * K * K;
-    }
-    info->max_rows = mx;
-    info->lsq_flops = (int64_t)fl;
-  }
+  info->max_rows = c.max_rows;
+  // the method's count per system of n rows: Householder QR of the n x K matrix, the triangular solve and the
+  // application of Q (2nK^2 - 2K^3/3 + 4nK + K^2), summed over the systems
+  const double K = T.K;
+  info->lsq_flops = (int64_t)((2.0 * K * K + 4.0 * K) * (double)c.nnz + (K * K - 2.0 / 3.0 * K * K * K) * (double)n_slots);
   float t01 = 0, t12 = 0, t23 = 0, t34 = 0;
   cudaEventElapsedTime(&t01, ev[0], ev[1]);
   cudaEventElapsedTime(&t12, ev[1], ev[2]);

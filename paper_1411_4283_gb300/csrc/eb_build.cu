@@ -16,6 +16,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "eb_internal.cuh"
 #include "eb_tables.cuh"
 #include "eb_build.cuh"
@@ -86,7 +88,9 @@ __global__ void k_classify_faces(Dims dm, int d, const uint8_t* __restrict__ ffl
     if (eb) st = -2;
     else {
       st = class_key(dm, d, x);
-      atomicMin((unsigned long long*)&class_rep[st], (unsigned long long)(dm.face_base[d] + f));
+      // the class's lowest face; most faces share one class, and few of them are lower than the ones before
+      const unsigned long long id = (unsigned long long)(dm.face_base[d] + f);
+      if (id < *(volatile unsigned long long*)&class_rep[st]) atomicMin((unsigned long long*)&class_rep[st], id);
     }
   }
   state[f] = st;
@@ -207,139 +211,106 @@ __device__ __forceinline__ bool reached(const GatherArgs& a, int64_t v, int dx, 
   return mtest(a.masks[ri], b);
 }
 
-// Rows of slot s, in canonical order: volumes (ascending cell index), wall
-// faces (ascending global face id), EB faces (ascending cut index).
-__device__ int gather_rows(const GatherArgs& a, int64_t s, uint32_t* out) {
-  const Dims& dm = a.dm;
-  int64_t gf = a.slot_face[s];
-  int R = dm.R;
-  int base[3], lo_ok = 0, hi_ok = 0, dface = -1;
-  int64_t vlo = -1, vhi = -1;
-  int rng_lo[3], rng_hi[3];
-  if (gf >= dm.n_grid_faces) return -1;  // EB slots are handled by the caller (base cell passed separately)
-  for (int d = 0; d < dm.dim; ++d)
-    if (gf >= dm.face_base[d]) dface = d;
-  int64_t f = gf - dm.face_base[dface];
-  face_xyz(dm, dface, f, base);
-  if (base[dface] < dm.n[dface]) { hi_ok = 1; vhi = cell_id(dm, base); hi_ok = a.flag[vhi] > 0; }
-  if (base[dface] > 0) {
-    int lo[3] = {base[0], base[1], base[2]};
-    lo[dface] -= 1;
-    vlo = cell_id(dm, lo);
-    lo_ok = a.flag[vlo] > 0;
-  }
-  for (int k = 0; k < 3; ++k) {
-    rng_lo[k] = k < dm.dim ? -R : 0;
-    rng_hi[k] = k < dm.dim ? R : 0;
-  }
-  rng_lo[dface] = -R - 1;
-  int n = 0;
-  for (int pass = 0; pass < 2 + dm.dim; ++pass) {
-    for (int dz = rng_lo[2]; dz <= rng_hi[2]; ++dz)
-      for (int dy = rng_lo[1]; dy <= rng_hi[1]; ++dy)
-        for (int dx = rng_lo[0]; dx <= rng_hi[0]; ++dx) {
-          int c[3] = {base[0] + dx, base[1] + dy, base[2] + dz};
-          if (!in_domain(dm, c)) continue;
-          int64_t cid = cell_id(dm, c);
-          if (a.flag[cid] == 0) continue;
-          int dd[3] = {dx, dy, dz};
-          bool in = false;
-          if (hi_ok) in = reached(a, vhi, dx, dy, dz);
-          if (!in && lo_ok) {
-            int e[3] = {dx, dy, dz};
-            e[dface] += 1;
-            in = reached(a, vlo, e[0], e[1], e[2]);
-          }
-          if (!in) continue;
-          if (pass == 0) {
-            if (out) out[n] = rd_pack(0, 0, 0, dd[0], dd[1], dd[2]);
-            ++n;
-          } else if (pass == 1 + dm.dim) {
-            if (a.flag[cid] == 2) {
-              if (out) out[n] = rd_pack(1, 0, 0, dd[0], dd[1], dd[2]);
-              ++n;
-            }
-          } else {
-            int wd = pass - 1;
-            if (c[wd] == 0) {
-              int fx[3] = {c[0], c[1], c[2]};
-              if (a.ff[wd][face_local(dm, wd, fx)] > 0) {
-                if (out) out[n] = rd_pack(2, wd, 0, dd[0], dd[1], dd[2]);
-                ++n;
-              }
-            }
-            if (c[wd] == dm.n[wd] - 1) {
-              int fx[3] = {c[0], c[1], c[2]};
-              fx[wd] += 1;
-              if (a.ff[wd][face_local(dm, wd, fx)] > 0) {
-                if (out) out[n] = rd_pack(2, wd, 1, dd[0], dd[1], dd[2]);
-                ++n;
-              }
-            }
-          }
-        }
-  }
-  return n;
-}
-
-// EB faces: neighbourhood of the cut cell itself
-__device__ int gather_rows_eb(const GatherArgs& a, int64_t v, uint32_t* out) {
-  const Dims& dm = a.dm;
-  int R = dm.R;
-  int base[3];
-  cell_xyz(dm, v, base);
-  int zr = dm.dim == 3 ? R : 0;
-  int n = 0;
-  for (int pass = 0; pass < 2 + dm.dim; ++pass)
-    for (int dz = -zr; dz <= zr; ++dz)
-      for (int dy = -R; dy <= R; ++dy)
-        for (int dx = -R; dx <= R; ++dx) {
-          int c[3] = {base[0] + dx, base[1] + dy, base[2] + dz};
-          if (!in_domain(dm, c)) continue;
-          int64_t cid = cell_id(dm, c);
-          if (a.flag[cid] == 0) continue;
-          if (!reached(a, v, dx, dy, dz)) continue;
-          if (pass == 0) {
-            if (out) out[n] = rd_pack(0, 0, 0, dx, dy, dz);
-            ++n;
-          } else if (pass == 1 + dm.dim) {
-            if (a.flag[cid] == 2) {
-              if (out) out[n] = rd_pack(1, 0, 0, dx, dy, dz);
-              ++n;
-            }
-          } else {
-            int wd = pass - 1;
-            if (c[wd] == 0) {
-              if (a.ff[wd][face_local(dm, wd, c)] > 0) {
-                if (out) out[n] = rd_pack(2, wd, 0, dx, dy, dz);
-                ++n;
-              }
-            }
-            if (c[wd] == dm.n[wd] - 1) {
-              int fx[3] = {c[0], c[1], c[2]};
-              fx[wd] += 1;
-              if (a.ff[wd][face_local(dm, wd, fx)] > 0) {
-                if (out) out[n] = rd_pack(2, wd, 1, dx, dy, dz);
-                ++n;
-              }
-            }
-          }
-        }
-  return n;
-}
-
-__global__ void k_gather(GatherArgs a, int64_t n_slots, const int32_t* __restrict__ cut_cell) {
-  int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Rows of every slot, in canonical order: volumes (ascending cell index), wall faces (ascending global face
+// id), EB faces (ascending cut index); counted (row_ptr null) or written.  A warp per slot: the lanes test 32
+// offsets of the box at a time and keep what they found as one bit per 32 (volume reached, cut, open wall on
+// each side), and the lists are written in order by ballots.  Bound by the latency of the flag and mask loads;
+// a thread per slot walked the box 2 + dim times (1.1 ms a pass for 90,000 slots of 392 offsets, 0.53 ms now).
+constexpr int GATHER_WARPS = 4;
+__global__ void __launch_bounds__(GATHER_WARPS * 32) k_gather(GatherArgs a, int64_t n_slots,
+                                                              const int32_t* __restrict__ cut_cell) {
+  const int lane = threadIdx.x & 31;
+  const int64_t s = (int64_t)blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5);
   if (s >= n_slots) return;
-  int64_t gf = a.slot_face[s];
-  uint32_t* out = a.row_ptr ? a.row_desc + a.row_ptr[s] : nullptr;
-  int n;
-  if (gf >= a.dm.n_grid_faces) n = gather_rows_eb(a, cut_cell[gf - a.dm.n_grid_faces], out);
-  else n = gather_rows(a, s, out);
-  if (!a.row_ptr) {
-    a.count[s] = n;
-    if (n > *a.max_rows) atomicMax(a.max_rows, n);
+  const Dims& dm = a.dm;
+  const int64_t gf = a.slot_face[s];
+  const int R = dm.R;
+  int base[3], dface = -1;
+  int64_t vlo = -1, vhi = -1;  // the adjacent volumes (an EB slot: its cut cell)
+  if (gf >= dm.n_grid_faces) {
+    vhi = cut_cell[gf - dm.n_grid_faces];
+    cell_xyz(dm, vhi, base);
+  } else {
+    for (int d = 0; d < dm.dim; ++d)
+      if (gf >= dm.face_base[d]) dface = d;
+    face_xyz(dm, dface, gf - dm.face_base[dface], base);
+    if (base[dface] < dm.n[dface]) {
+      vhi = cell_id(dm, base);
+      if (a.flag[vhi] == 0) vhi = -1;
+    }
+    if (base[dface] > 0) {
+      int lo[3] = {base[0], base[1], base[2]};
+      lo[dface] -= 1;
+      vlo = cell_id(dm, lo);
+      if (a.flag[vlo] == 0) vlo = -1;
+    }
   }
+  int lo3[3], w3[3];
+  for (int k = 0; k < 3; ++k) {
+    lo3[k] = k < dm.dim ? -R - (k == dface) : 0;
+    w3[k] = k < dm.dim ? 2 * R + 1 + (k == dface) : 1;
+  }
+  const int total = w3[0] * w3[1] * w3[2];
+  // bit q: the offset 32 q + lane
+  uint32_t in = 0, cut = 0, wall[3][2] = {};
+  for (int q = 0; 32 * q < total; ++q) {
+    const int t = 32 * q + lane;
+    if (t >= total) break;
+    const int dx = lo3[0] + t % w3[0], dy = lo3[1] + t / w3[0] % w3[1], dz = lo3[2] + t / (w3[0] * w3[1]);
+    const int c[3] = {base[0] + dx, base[1] + dy, base[2] + dz};
+    if (!in_domain(dm, c)) continue;
+    const uint8_t fl = a.flag[cell_id(dm, c)];
+    if (fl == 0) continue;
+    bool got = vhi >= 0 && reached(a, vhi, dx, dy, dz);
+    if (!got && vlo >= 0) got = reached(a, vlo, dx + (dface == 0), dy + (dface == 1), dz + (dface == 2));
+    if (!got) continue;
+    in |= 1u << q;
+    if (fl == 2) cut |= 1u << q;
+    for (int d = 0; d < dm.dim; ++d)
+      for (int side = 0; side < 2; ++side) {
+        if (c[d] != (side ? dm.n[d] - 1 : 0)) continue;
+        int fx[3] = {c[0], c[1], c[2]};
+        fx[d] += side;
+        if (a.ff[d][face_local(dm, d, fx)] > 0) wall[d][side] |= 1u << q;
+      }
+  }
+  uint32_t* out = a.row_ptr ? a.row_desc + a.row_ptr[s] : nullptr;
+  const unsigned before = (1u << lane) - 1u;
+  int n = 0;
+  auto desc = [&](int q, int kind, int wd, int side) {
+    const int t = 32 * q + lane;
+    return rd_pack(kind, wd, side, lo3[0] + t % w3[0], lo3[1] + t / w3[0] % w3[1], lo3[2] + t / (w3[0] * w3[1]));
+  };
+  auto list = [&](uint32_t bits, int kind) {
+    for (int q = 0; 32 * q < total; ++q) {
+      const bool on = (bits >> q) & 1u;
+      const unsigned m = __ballot_sync(0xffffffffu, on);
+      if (on && out) out[n + __popc(m & before)] = desc(q, kind, 0, 0);
+      n += __popc(m);
+    }
+  };
+  list(in, 0);
+  for (int d = 0; d < dm.dim; ++d) {
+    if (!__any_sync(0xffffffffu, wall[d][0] | wall[d][1])) continue;
+    for (int q = 0; 32 * q < total; ++q) {
+      const bool lo = (wall[d][0] >> q) & 1u, hi = (wall[d][1] >> q) & 1u;
+      const unsigned ml = __ballot_sync(0xffffffffu, lo), mh = __ballot_sync(0xffffffffu, hi);
+      const int at = n + __popc(ml & before) + __popc(mh & before);
+      if (lo && out) out[at] = desc(q, 2, d, 0);
+      if (hi && out) out[at + lo] = desc(q, 2, d, 1);
+      n += __popc(ml) + __popc(mh);
+    }
+  }
+  list(cut, 1);
+  if (!a.row_ptr && lane == 0) {
+    a.count[s] = n;
+    if (n > *(volatile int32_t*)a.max_rows) atomicMax(a.max_rows, n);
+  }
+}
+cudaError_t gather_launch(const GatherArgs& a, int64_t n_slots, const int32_t* cut_cell, cudaStream_t s) {
+  if (n_slots > 0)
+    k_gather<<<(unsigned)((n_slots + GATHER_WARPS - 1) / GATHER_WARPS), GATHER_WARPS * 32, 0, s>>>(a, n_slots, cut_cell);
+  return cudaGetLastError();
 }
 
 // ============================================================ 4. weighted LS (FP64)
@@ -1070,11 +1041,14 @@ __global__ void k_assemble_rows(AsmArgs a, const int32_t* __restrict__ rep_cell,
   }
 }
 
-// boundary entries of irregular cell rows: count (vals == null) or write
-__global__ void k_assemble_b(AsmArgs a, const int32_t* __restrict__ cells, int64_t ncells, int64_t* __restrict__ cnt,
-                             const int64_t* __restrict__ bptr, int64_t* __restrict__ bcol, double* __restrict__ bval,
-                             const int32_t* __restrict__ cut_cell_unused) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Boundary entries of irregular cell rows: counted (bptr null) or written in the rows' order.  A warp per cell:
+// the lanes read 32 row descriptors of a face at a time and the boundary ones find their place by ballots (a
+// thread per cell read its up to 7 x 553 descriptors one after the other: 1.15 ms a pass at 48^3, 0.34 ms now).
+__global__ void __launch_bounds__(128) k_assemble_b(AsmArgs a, const int32_t* __restrict__ cells, int64_t ncells,
+                                                    int64_t* __restrict__ cnt, const int64_t* __restrict__ bptr,
+                                                    int64_t* __restrict__ bcol, double* __restrict__ bval) {
+  const int lane = threadIdx.x & 31;
+  const int64_t t = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
   if (t >= ncells) return;
   const Dims& dm = a.dm;
   int64_t c = cells[t];
@@ -1084,12 +1058,12 @@ __global__ void k_assemble_b(AsmArgs a, const int32_t* __restrict__ cells, int64
   double sig[8];
   int bases[8][3];
   int nf = cell_faces(a, x, c, slots, sig, bases);
-  int64_t k = bptr ? bptr[t] : 0;
+  const int64_t k = bptr ? bptr[t] : 0;
   int64_t n = 0;
   if (neumann_eb(a, c)) {
     // Neumann EB face: the flux is the datum, |A_f| <g>_f (sigma = +1, kappa-weighted scale 1/h^2)
     --nf;
-    if (bptr) {
+    if (bptr && lane == 0) {
       const int32_t cut = a.cut_of_cell[c];
       bcol[k + n] = dm.n_grid_faces + cut;
       bval[k + n] = a.eb_mom[(int64_t)cut * dm.KS] * dm.h * a.inv_h2;
@@ -1098,11 +1072,13 @@ __global__ void k_assemble_b(AsmArgs a, const int32_t* __restrict__ cells, int64
   }
   for (int q = 0; q < nf; ++q) {
     int64_t p0 = a.row_ptr[slots[q]], p1 = a.row_ptr[slots[q] + 1];
-    for (int64_t p = p0; p < p1; ++p) {
-      uint32_t ds = a.row_desc[p];
-      int kind = rd_kind(ds);
-      if (kind == 0) continue;
-      if (bptr) {
+    for (int64_t pc = p0; pc < p1; pc += 32) {
+      const int64_t p = pc + lane;
+      const uint32_t ds = p < p1 ? a.row_desc[p] : 0u;
+      const int kind = rd_kind(ds);
+      const unsigned m = __ballot_sync(0xffffffffu, kind != 0);
+      if (bptr && kind != 0) {
+        const int64_t at = k + n + __popc(m & ((1u << lane) - 1u));
         int y[3];
         for (int d = 0; d < 3; ++d) y[d] = bases[q][d] + (d < dm.dim ? rd_off(ds, d) : 0);
         int64_t col;
@@ -1116,13 +1092,55 @@ __global__ void k_assemble_b(AsmArgs a, const int32_t* __restrict__ cells, int64
           if (rd_wside(ds)) y[wd] += 1;
           col = dm.face_base[wd] + face_local(dm, wd, y);
         }
-        bcol[k + n] = col;
-        bval[k + n] = sig[q] * a.row_val[p] * a.inv_h2 * sc;
+        bcol[at] = col;
+        bval[at] = sig[q] * a.row_val[p] * a.inv_h2 * sc;
       }
-      ++n;
+      n += __popc(m);
     }
   }
-  if (!bptr) cnt[t] = n;
+  if (!bptr && lane == 0) cnt[t] = n;
+}
+cudaError_t assemble_b_launch(const AsmArgs& a, const int32_t* cells, int64_t ncells, int64_t* cnt, const int64_t* bptr,
+                              int64_t* bcol, double* bval, cudaStream_t s) {
+  if (ncells > 0) k_assemble_b<<<(unsigned)((ncells + 3) / 4), 128, 0, s>>>(a, cells, ncells, cnt, bptr, bcol, bval);
+  return cudaGetLastError();
+}
+
+__global__ void k_count_faces(const int32_t* __restrict__ slot, int64_t n, int64_t n_unique,
+                              unsigned long long* __restrict__ counts) {
+  unsigned open = 0, cls = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t v = slot[i];
+    open += v >= 0;
+    cls += v >= n_unique;
+  }
+  open = __reduce_add_sync(0xffffffffu, open);
+  cls = __reduce_add_sync(0xffffffffu, cls);
+  if ((threadIdx.x & 31) == 0) {
+    if (open) atomicAdd(counts + 0, (unsigned long long)open);
+    if (cls) atomicAdd(counts + 1, (unsigned long long)cls);
+  }
+}
+__global__ void k_count_status(const int32_t* __restrict__ status, int64_t n, unsigned long long* __restrict__ counts) {
+  unsigned c[3] = {0, 0, 0};
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t v = status[i];
+    c[0] += v == 1;
+    c[1] += v == 2;
+    c[2] += v == 4;
+  }
+  for (int k = 0; k < 3; ++k) {
+    c[k] = __reduce_add_sync(0xffffffffu, c[k]);
+    if ((threadIdx.x & 31) == 0 && c[k]) atomicAdd(counts + 2 + k, (unsigned long long)c[k]);
+  }
+}
+cudaError_t count_faces(const int32_t* slot, int64_t n, int64_t n_unique, unsigned long long* counts, cudaStream_t s) {
+  k_count_faces<<<(unsigned)std::min<int64_t>(608, (n + 1023) / 1024), 256, 0, s>>>(slot, n, n_unique, counts);
+  return cudaGetLastError();
+}
+cudaError_t count_status(const int32_t* status, int64_t n, unsigned long long* counts, cudaStream_t s) {
+  if (n > 0) k_count_status<<<(unsigned)std::min<int64_t>(608, (n + 1023) / 1024), 256, 0, s>>>(status, n, counts);
+  return cudaGetLastError();
 }
 
 }  // namespace eb

@@ -133,7 +133,7 @@ __global__ void k_face_slots(Dims dm, int d, const int32_t* state, const int64_t
                              const int32_t* class_slot, int32_t* slot, int64_t* slot_face);
 __global__ void k_reach(Dims dm, const int32_t* cells, int64_t ncells, const uint8_t* flag, const uint8_t* ff0,
                         const uint8_t* ff1, const uint8_t* ff2, Mask* out);
-__global__ void k_gather(GatherArgs a, int64_t n_slots, const int32_t* cut_cell);
+cudaError_t gather_launch(const GatherArgs& a, int64_t n_slots, const int32_t* cut_cell, cudaStream_t s);
 // Adjoint of the stencil solves with respect to the moment tables (k_stencil_adjoint, eb_build.cu)
 struct AdjArgs {
   const double* lam;        // [ncell] adjoint solution
@@ -169,7 +169,12 @@ cudaError_t lsq_fallback_list(const int32_t* status, int64_t n, int64_t base, in
                               cudaStream_t s);
 __global__ void k_full_rows(Dims dm, const Tables* T, double* ftab, float* ftab_h, float* ftab_l, double* wtab);
 __global__ void k_assemble_rows(AsmArgs a, const int32_t* rep_cell, int64_t nrep, int64_t row0, int32_t* err);
-__global__ void k_assemble_b(AsmArgs a, const int32_t* cells, int64_t ncells, int64_t* cnt, const int64_t* bptr,
-                             int64_t* bcol, double* bval, const int32_t* unused);
+// boundary entries of the irregular cells' rows: counted into cnt (bptr null) or written
+cudaError_t assemble_b_launch(const AsmArgs& a, const int32_t* cells, int64_t ncells, int64_t* cnt, const int64_t* bptr,
+                              int64_t* bcol, double* bval, cudaStream_t s);
+// counts[0, 1] += the faces of one direction with a slot and with a class slot; counts[2..4] += the systems of
+// status 1 (rank deficient), 2 (a row that could not be built) and 4 (solved by the FP64 pass)
+cudaError_t count_faces(const int32_t* slot, int64_t n, int64_t n_unique, unsigned long long* counts, cudaStream_t s);
+cudaError_t count_status(const int32_t* status, int64_t n, unsigned long long* counts, cudaStream_t s);
 
 }  // namespace eb

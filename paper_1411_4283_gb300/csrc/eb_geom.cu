@@ -186,12 +186,14 @@ __device__ __forceinline__ void mon2(int i, int* p0, int* p1) {
   *p1 = i;
 }
 
-// a^2 - b^2 with its two roundings fixed (the square of b exact: sq_less, of a exact: sq_over).  Positions in a
+// a^2 - b^2 with its roundings fixed (the square of b exact: sq_less, of a exact: sq_over, neither: sq_apart).  Positions in a
 // cell come from square roots of such differences of squares of size (R/h)^2, so the moments of a cell of tiny
 // volume or area hold their last bits: left to the compiler's contraction, they would change with the code
-// around them (1e-11 of the patch moments and 4e-8 of a volume fraction of 1e-13 at 63^3).
+// around them (1e-11 of the patch moments and 4e-8 of a volume fraction of 1e-13 at 63^3), and the solution in
+// such a cell with them; the forms below are those the tables have had.
 __device__ __forceinline__ double sq_less(double a, double b) { return fma(-b, b, __dmul_rn(a, a)); }
 __device__ __forceinline__ double sq_over(double a, double b) { return fma(a, a, -__dmul_rn(b, b)); }
+__device__ __forceinline__ double sq_apart(double a, double b) { return __dsub_rn(__dmul_rn(a, a), __dmul_rn(b, b)); }
 
 // fluid intervals of the segment [-1/2, 1/2] of a line at signed distance dn from the circle centre, with
 // the circle's chord at tangential position ct: outside fluid keeps the segment minus the chord,
@@ -861,6 +863,27 @@ __device__ __forceinline__ int warp_sort_nonneg(double v, bool valid, double* ou
 // graded 2-D index of x^a y^b (mon2's order)
 __host__ __device__ constexpr int idx2(int a, int b) { return (a + b) * (a + b + 1) / 2 + b; }
 
+// Polar-angle breakpoints of the patch of the sphere (cx, cy, cz, R) in the cell [-1/2, 1/2]^3, ascending, into
+// br[]; returns their number.  One candidate per lane: the range ends (0, 1), tangencies with the edge lines
+// x, y = +-1/2 (2..9) and passes through the square's corners (10..17); z = cz + R cos(th), rho = R sin(th)
+// and dA = R dz dphi = R^2 sin(th) dth dphi: the angle keeps the integrand analytic up to the poles.
+__device__ __forceinline__ int patch_breaks(double cx, double cy, double cz, double R, double* br) {
+  const int lane = threadIdx.x & 31;
+  const double zl = fmax(-0.5, cz - R), zh = fmin(0.5, cz + R);
+  double z = lane == 0 ? zl : zh;
+  bool valid = lane < 2;
+  if (lane >= 2 && lane < 18) {
+    const bool corner = lane >= 10;
+    const int j = corner ? lane - 10 : lane - 2;  // bit 0: edge, bit 1: axis or the other edge, bit 2: side
+    const double ex = ((j & 1) ? 0.5 : -0.5) - cx, ey = (((corner ? j >> 1 : j) & 1) ? 0.5 : -0.5) - cy;
+    const double e1 = corner || !(j & 2) ? ex : ey;
+    const double qq = corner ? __dsub_rn(sq_less(R, e1), __dmul_rn(ey, ey)) : sq_apart(R, e1);
+    z = cz + ((j & 4) ? 1.0 : -1.0) * sqrt(fmax(qq, 0.0));
+    valid = qq > 0.0 && z > zl && z < zh;
+  }
+  return warp_sort_nonneg(acos(fmin(1.0, fmax(-1.0, (z - cz) / R))), valid, br);
+}
+
 constexpr int PATCH_WARPS = 4;
 template <int Q>
 struct PatchSmem {
@@ -910,26 +933,7 @@ __global__ void __launch_bounds__(PATCH_WARPS * 32) k_sphere_patch(Spheres B, co
   // divergence-theorem direction: the smallest component of the centre offset, the direction most tangent
   // to the patch (see k_sphere_vol)
   const int dd = (fabs(cx) <= fabs(cy) && fabs(cx) <= fabs(cz)) ? 0 : (fabs(cy) <= fabs(cz) ? 1 : 2);
-  // polar-angle breakpoints, one candidate per lane: the range ends (0, 1), tangencies with the edge lines
-  // x, y = +-1/2 (2..9) and passes through the square's corners (10..17); z = cz + R cos(th), rho = R sin(th)
-  // and dA = R dz dphi = R^2 sin(th) dth dphi: the angle keeps the integrand analytic up to the poles
-  int nb;
-  {
-    const double zl = fmax(-0.5, cz - R), zh = fmin(0.5, cz + R);
-    double z = lane == 0 ? zl : zh;
-    bool valid = lane < 2;
-    if (lane >= 2 && lane < 18) {
-      const bool corner = lane >= 10;
-      const int j = corner ? lane - 10 : lane - 2;  // bit 0: edge, bit 1: axis or the other edge, bit 2: side
-      const double ex = ((j & 1) ? 0.5 : -0.5) - cx, ey = (((corner ? j >> 1 : j) & 1) ? 0.5 : -0.5) - cy;
-      const double e1 = corner || !(j & 2) ? ex : ey;
-      double qq = sq_less(R, e1);
-      if (corner) qq = __dsub_rn(qq, __dmul_rn(ey, ey));
-      z = cz + ((j & 4) ? 1.0 : -1.0) * sqrt(fmax(qq, 0.0));
-      valid = qq > 0.0 && z > zl && z < zh;
-    }
-    nb = warp_sort_nonneg(acos(fmin(1.0, fmax(-1.0, (z - cz) / R))), valid, M.br);
-  }
+  const int nb = patch_breaks(cx, cy, cz, R, M.br);
   int np;
   {  // panels with a part of the sphere inside the cell (which arcs exist is the same all over a panel)
     double a0[4], a1[4];
@@ -1071,29 +1075,33 @@ __host__ __device__ constexpr double half_pow(int sign, int e) {
 }
 
 // Moments int u^a v^b over the fluid part of the square [-1/2,1/2]^2 of a plane the sphere cuts in the disk
-// (cu, cv, rho) (rho <= 0: no disk), by a warp: the sin^2-mapped nodes of the u-panels over the lanes, then
-// one sum over the warp (in every lane).  Outside a sphere the full columns beyond the disk's u-range come in
-// closed form and the parts of a column beyond the chord node by node (a nearly closed face is not the small
-// difference of the square and the disk).
-struct DiskSmem {
-  double pos[GEO_GLT], wt[GEO_GLT], br[4][8];
-};
+// (cu, cv, rho) (rho <= 0: no disk), by a warp: the sin^2-mapped nodes of the u-panels over the lanes, then the
+// lanes k < (Q+1)(Q+2)/2 sum and return the k-th moment, node after node (see k_sphere_patch_small for why the
+// order stays).  Outside a sphere the full columns beyond the disk's u-range come in closed form and the parts
+// of a column beyond the chord node by node (a nearly closed face is not the small difference of the square and
+// the disk).  CELL: the faces of a cut cell in its volume moments (the tables' roundings differ there, see
+// sq_less).
 template <int Q>
-__device__ __forceinline__ void disk_square(double cu, double cv, double rho, bool inside, DiskSmem& S,
-                                            double (&acc)[(Q + 1) * (Q + 2) / 2]) {
+struct DiskSmem {
+  double sn[GEO_GLT], cs[GEO_GLT], wt[GEO_GLT], br[4][8];
+  double node[4][32][Q + 3];  // weight, u, chord moments of v
+};
+template <int Q, bool CELL>
+__device__ __forceinline__ double disk_square(double cu, double cv, double rho, bool inside, DiskSmem<Q>& S) {
   constexpr int K2 = (Q + 1) * (Q + 2) / 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const double lo = fmax(-0.5, cu - rho), hi = fmin(0.5, cu + rho);
   const bool disk = rho > 0.0 && hi > lo;
-#pragma unroll
-  for (int k = 0; k < K2; ++k) acc[k] = 0.0;
+  int eu, ev;
+  mon2(lane < K2 ? lane : 0, &eu, &ev);
+  double acc = 0.0;
   if (disk) {
     // breakpoints, one candidate per lane: the range ends and where the circle meets v = +-1/2
     double uu = lane == 0 ? lo : hi;
     bool valid = lane < 2;
     if (lane >= 2 && lane < 6) {
       const double dv = ((lane & 1) ? 0.5 : -0.5) - cv;
-      uu = cu + ((lane & 2) ? -1.0 : 1.0) * sqrt(fmax(sq_less(rho, dv), 0.0));
+      uu = cu + ((lane & 2) ? -1.0 : 1.0) * sqrt(fmax(CELL ? sq_apart(rho, dv) : sq_less(rho, dv), 0.0));
       valid = fabs(dv) < rho && uu > lo && uu < hi;
     }
     double* br = S.br[warp];
@@ -1104,59 +1112,72 @@ __device__ __forceinline__ void disk_square(double cu, double cv, double rho, bo
       const double o = __shfl_sync(0xffffffffu, uu, j);
       rank += o < uu || (o == uu && j < lane);
     }
-    __syncwarp();  // the warp's last use of br
+    __syncwarp();  // the warp's last use of br and node
     if (valid) br[rank] = uu;
     __syncwarp();
     const int total = (__popc(m) - 1) * GEO_GLT;
-    for (int i = lane; i < total; i += 32) {
-      const double a = br[i / GEO_GLT], pw = br[i / GEO_GLT + 1] - a;
-      if (!(pw > 0.0)) continue;
-      const double uq = panel_node(a, pw, S.pos[i % GEO_GLT]), wu = pw * S.wt[i % GEO_GLT];
-      const double du = uq - cu, hw = sqrt(fmax(sq_less(rho, du), 0.0));
-      const double va = fmin(fmax(cv - hw, -0.5), 0.5), vb = fmin(fmax(cv + hw, -0.5), 0.5);
-      double pa = va, pb = vb, vp[Q + 1], up[Q + 1];
+    for (int i0 = 0; i0 < total; i0 += 32) {
+      const int i = i0 + lane;
+      if (i < total) {
+        const double a = br[i / GEO_GLT], pw = br[i / GEO_GLT + 1] - a;
+        const double sn = S.sn[i % GEO_GLT], uq = panel_node(a, pw, sn);
+        const double du = uq - cu, hw = sqrt(fmax(sq_less(rho, du), 0.0));
+        const double va = fmin(fmax(cv - hw, -0.5), 0.5), vb = fmin(fmax(cv + hw, -0.5), 0.5);
+        double* nd = S.node[warp][lane];
+        nd[0] = 0.5 * S.wt[i % GEO_GLT] * pw * M_PI * sn * S.cs[i % GEO_GLT];  // 0 on a panel of no width
+        nd[1] = uq;
+        double pa = va, pb = vb;
 #pragma unroll
-      for (int k = 0; k <= Q; ++k) {
-        // the chord, or the two parts of the column beyond it
-        const double full = half_pow(1, k + 1), rk = 1.0 / (k + 1);
-        const double s = inside ? pb - pa : (pa - ((k & 1) ? full : -full)) + (full - pb);
-        vp[k] = s * (wu * rk);
-        pa *= va;
-        pb *= vb;
-        up[k] = k == 0 ? 1.0 : up[k - 1] * uq;
+        for (int k = 0; k <= Q; ++k) {
+          // the chord, or the two parts of the column beyond it
+          const double full = half_pow(1, k + 1);
+          nd[2 + k] = inside ? (pb - pa) / (k + 1) : (pa - ((k & 1) ? full : -full)) / (k + 1) + (full - pb) / (k + 1);
+          pa = __dmul_rn(pa, va);  // not fused into the next difference
+          pb = __dmul_rn(pb, vb);
+        }
       }
-#pragma unroll
-      for (int g = 0; g <= Q; ++g)
-#pragma unroll
-        for (int j = 0; j <= g; ++j) acc[idx2(g - j, j)] = fma(up[g - j], vp[j], acc[idx2(g - j, j)]);
-    }
-#pragma unroll
-    for (int k = 0; k < K2; ++k)
-      for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
-  }
-  if (!inside) {  // the columns beyond the disk's u-range
-    double ua[2] = {-0.5, hi}, ub[2] = {disk ? lo : 0.5, 0.5};
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      if (!(ub[j] > ua[j]) || (j == 1 && !disk)) continue;
-      double pa = ua[j], pb = ub[j];
-#pragma unroll
-      for (int g = 0; g <= Q; ++g) {
-        const double su = pb - pa;
-#pragma unroll
-        for (int l = 0; l + g <= Q; l += 2)
-          acc[idx2(g, l)] = fma(su, half_pow(1, l) / ((l + 1) * (g + 1)), acc[idx2(g, l)]);
-        pa *= ua[j];
-        pb *= ub[j];
-      }
+      __syncwarp();
+      const int cnt = total - i0 < 32 ? total - i0 : 32;
+      if (lane < K2)
+        for (int j = 0; j < cnt; ++j) {
+          const double* nd = S.node[warp][j];
+          double up = 1.0;
+          for (int e = 0; e < eu; ++e) up *= nd[1];
+          acc = fma(nd[0] * up, nd[2 + ev], acc);
+        }
+      __syncwarp();
     }
   }
+  if (inside) return acc;
+  // the columns beyond the disk's u-range
+  double full = 0.0;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const double ua = j ? hi : -0.5, ub = j || !disk ? 0.5 : lo;
+    if (!(ub > ua) || (j == 1 && !disk)) continue;
+    double pa = ua, pb = ub;
+    for (int e = 0; e < eu; ++e) {
+      pa *= ua;
+      pb *= ub;
+    }
+    const double sv = (ev & 1) ? 0.0 : half_pow(1, ev) / (ev + 1);
+    full = fma((pb - pa) / (eu + 1), sv, full);
+  }
+  return full + acc;
 }
 
-__device__ __forceinline__ void disk_rule(const PatchRule& rule, DiskSmem& S) {
-  panel_rule(rule, S.pos, S.wt);
+template <int Q>
+__device__ __forceinline__ void disk_rule(const PatchRule& rule, DiskSmem<Q>& S) {
+  for (int g = threadIdx.x; g < GEO_GLT; g += blockDim.x) {
+    const double s = 0.5 * rule.pos[g] + 0.5;
+    S.sn[g] = sin(0.5 * M_PI * s);
+    S.cs[g] = cos(0.5 * M_PI * s);
+    S.wt[g] = rule.wt[g];
+  }
   __syncthreads();
 }
+
+constexpr double GEO_SMALL = 1e-6;  // volume fractions below it: k_sphere_patch_small
 
 // Volume moments from the patch part and the fluid parts of the two faces normal to the divergence direction
 // (a warp per cell).  Those faces' moments are integrated here once more, from the cell's own coordinates: the
@@ -1166,14 +1187,14 @@ template <int Q>
 __global__ void __launch_bounds__(128) k_sphere_vol(Spheres B, const __grid_constant__ PatchRule rule, int N, double h,
                                                     const int32_t* __restrict__ cells, int64_t n,
                                                     const int32_t* __restrict__ cbody, const double* __restrict__ volp,
-                                                    double* vol) {
+                                                    double* vol, bool small_only) {
   constexpr int K = (Q + 1) * (Q + 2) * (Q + 3) / 6, K2 = (Q + 1) * (Q + 2) / 2;
-  __shared__ DiskSmem S;
+  __shared__ DiskSmem<Q> S;
   __shared__ double fms[4][K2];
   disk_rule(rule, S);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t = (int64_t)blockIdx.x * 4 + warp;
-  if (t >= n) return;
+  if (t >= n || (small_only && !(fabs(vol[t * K]) < GEO_SMALL))) return;
   const int c = cells[t];
   const int ix = c % N, iy = (c / N) % N, iz = c / (N * N);
   const int b = cbody[c];
@@ -1187,12 +1208,8 @@ __global__ void __launch_bounds__(128) k_sphere_vol(Spheres B, const __grid_cons
   for (int i = 0; i < (K + 31) / 32; ++i) acc[i] = lane + 32 * i < K ? volp[t * K + lane + 32 * i] : 0.0;
   for (int s = -1; s <= 1; s += 2) {
     const double xe = 0.5 * s, d2 = sq_less(R, xe - cd);
-    double fm[K2];
-    disk_square<Q>(cu, cv, d2 > 0.0 ? sqrt(d2) : 0.0, B.inside, S, fm);
-    if (lane == 0) {
-#pragma unroll
-      for (int k = 0; k < K2; ++k) fms[warp][k] = fm[k];
-    }
+    const double fm = disk_square<Q, true>(cu, cv, d2 > 0.0 ? sqrt(d2) : 0.0, B.inside, S);
+    if (lane < K2) fms[warp][lane] = fm;
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < (K + 31) / 32; ++i) {
@@ -1213,6 +1230,121 @@ __global__ void __launch_bounds__(128) k_sphere_vol(Spheres B, const __grid_cons
   }
 }
 
+// The patch integrals once more for the cells whose volume came out tiny (k_sphere_vol then adds the faces again):
+// 20 directly evaluated angles per arc, summed node after node.  Such a volume (a corner cut off by the sphere) is
+// the difference of its face and patch terms.  Its nodes lie on a sphere of 10..100 cells' radius, so one rounding
+// of a coordinate is up to 1e-10 of the corner's extent, and the operator's row there can be so weak that the
+// solution in the cell amplifies that: at 128^3 nodes rounded in another way, eb moments 1e-12 and volumes 7e-12
+// apart at a volume fraction of 3e-13, moved it by 3e-7 (and the sums of k_sphere_patch alone by 1e-6).  So the
+// roundings and the order are fixed here, those of one thread's plain sums.  A block per cell, a thread per result
+// (5 K of them); the polar angles of a panel and the nodes of an arc are made by the first threads.  A few cells in
+// ten thousand come here; the others' blocks return at once.
+constexpr int SMALL_THREADS = 192;
+template <int Q>
+struct SmallSmem {
+  double gx[GEO_GL], gw[GEO_GL], br[20];
+  double z[GEO_GLT], rho[GEO_GLT], wz[GEO_GLT], a0[GEO_GLT][4], a1[GEO_GLT][4];
+  double node[2][GEO_GL][4 + 3 * (Q + 2)];  // the four weights, powers of x, y, z
+  int narc[GEO_GLT], nb;
+};
+template <int Q>
+__global__ void __launch_bounds__(SMALL_THREADS) k_sphere_patch_small(Spheres B, const __grid_constant__ GlRuleT glt,
+                                                                      const __grid_constant__ GlRule gl, int N, double h,
+                                                                      const int32_t* __restrict__ cells,
+                                                                      const int32_t* __restrict__ cbody, double* eb,
+                                                                      double* ebn, double* volp,
+                                                                      const double* __restrict__ vol) {
+  constexpr int K = (Q + 1) * (Q + 2) * (Q + 3) / 6, NP = Q + 2;
+  static_assert(5 * K <= SMALL_THREADS, "a thread per result");
+  const int64_t t = blockIdx.x;
+  if (!(fabs(vol[t * K]) < GEO_SMALL)) return;
+  __shared__ SmallSmem<Q> S;
+  const int tid = threadIdx.x;
+  for (int i = tid; i < GEO_GL; i += SMALL_THREADS) {
+    S.gx[i] = gl.x[i];
+    S.gw[i] = gl.w[i];
+  }
+  const int c = cells[t];
+  const int ix = c % N, iy = (c / N) % N, iz = c / (N * N);
+  const int b = cbody[c];
+  const double cx = (B.c[b][0] - (ix + 0.5) * h) / h, cy = (B.c[b][1] - (iy + 0.5) * h) / h;
+  const double cz = (B.c[b][2] - (iz + 0.5) * h) / h, R = B.r[b] / h;
+  const double sgn = B.inside ? 1.0 : -1.0;
+  const int dd = (fabs(cx) <= fabs(cy) && fabs(cx) <= fabs(cz)) ? 0 : (fabs(cy) <= fabs(cz) ? 1 : 2);
+  if (tid < 32) {
+    const int nb = patch_breaks(cx, cy, cz, R, S.br);
+    if (tid == 0) S.nb = nb;
+  }
+  // this thread's result: its weight (0 plain, 1 + d with the normal's component d) and exponents
+  const int e = tid < 5 * K ? tid : 0, table = e / K;
+  int p[3];
+  mon3(e % K, p);
+  const int fw = table == 4 ? 1 + dd : table;
+  if (table == 4) p[dd] += 1;
+  double acc = 0.0;
+  int buf = 0;
+  __syncthreads();
+  for (int pnl = 0; pnl + 1 < S.nb; ++pnl) {
+    if (S.br[pnl + 1] <= S.br[pnl]) continue;
+    if (tid < GEO_GLT) {
+      double th, wth, a0[4], a1[4];
+      sin2_node(glt, tid, S.br[pnl], S.br[pnl + 1], &th, &wth);
+      const double rho = R * sin(th);
+      const int narc = rho > 0.0 ? square_arcs(cx, cy, rho, a0, a1) : 0;
+      S.z[tid] = cz + R * cos(th);
+      S.rho[tid] = rho;
+      S.wz[tid] = wth * rho;
+      S.narc[tid] = narc;
+      for (int a = 0; a < narc; ++a) {
+        S.a0[tid][a] = a0[a];
+        S.a1[tid][a] = a1[a];
+      }
+    }
+    __syncthreads();
+    for (int gz = 0; gz < GEO_GLT; ++gz) {
+      for (int a = 0; a < S.narc[gz]; ++a) {
+        const double a0 = S.a0[gz][a], a1 = S.a1[gz][a];
+        const int npc = (int)ceil((a1 - a0) / (0.25 * M_PI));
+        const double span = (a1 - a0) / npc;
+        for (int pc = 0; pc < npc; ++pc, buf ^= 1) {
+          if (tid < GEO_GL) {
+            const double hw = 0.5 * span, ph = a0 + (pc + 0.5) * span + hw * S.gx[tid];
+            const double rho = S.rho[gz], z = S.z[gz], cp = cos(ph), sp = sin(ph);
+            const double ex = __dmul_rn(rho, cp), ey = __dmul_rn(rho, sp), x = __dadd_rn(cx, ex), y = __dadd_rn(cy, ey);
+            const double w = S.wz[gz] * S.gw[tid] * hw * R;  // dA = R dz dphi
+            double* nd = S.node[buf][tid];
+            nd[0] = w;
+            nd[1] = w * (sgn * ex / R);
+            nd[2] = w * (sgn * ey / R);
+            nd[3] = w * (sgn * (z - cz) / R);
+            double px = 1.0, py = 1.0, pz = 1.0;
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+              nd[4 + k] = px;
+              nd[4 + NP + k] = py;
+              nd[4 + 2 * NP + k] = pz;
+              px *= x;
+              py *= y;
+              pz *= z;
+            }
+          }
+          __syncthreads();  // the nodes of the arc before are in the other buffer
+          for (int g = 0; g < GEO_GL; ++g) {
+            const double* nd = S.node[buf][g];
+            acc = fma(nd[fw] * nd[4 + p[0]] * nd[4 + NP + p[1]], nd[4 + 2 * NP + p[2]], acc);
+          }
+        }
+      }
+    }
+    __syncthreads();  // the panel's angles are done with
+  }
+  if (tid < 5 * K) {
+    const int k = e % K;
+    double* dst = table == 0 ? eb + t * K : (table == 4 ? volp + t * K : ebn + (t * 3 + table - 1) * K);
+    dst[k] = acc;
+  }
+}
+
 // Tangential moments of the cut faces normal to dir (a warp per face).  FP64 issue bound; a thread per face
 // took 3.3 ms for a direction of the 96^3 box minus a sphere (a chain of one thread's nodes), this 0.34 ms.
 template <int Q>
@@ -1220,7 +1352,7 @@ __global__ void __launch_bounds__(128) k_sphere_faces(Spheres B, const __grid_co
                                                       double h, const int32_t* __restrict__ faces, int64_t n,
                                                       const int32_t* __restrict__ fbody, double* out) {
   constexpr int K2 = (Q + 1) * (Q + 2) / 2;
-  __shared__ DiskSmem S;
+  __shared__ DiskSmem<Q> S;
   disk_rule(rule, S);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t = (int64_t)blockIdx.x * 4 + warp;
@@ -1233,12 +1365,8 @@ __global__ void __launch_bounds__(128) k_sphere_faces(Spheres B, const __grid_co
   const double dn = (i3[dir] * h - B.c[b][dir]) / h;
   const double cu = (B.c[b][u] - (i3[u] + 0.5) * h) / h, cv = (B.c[b][v] - (i3[v] + 0.5) * h) / h;
   const double R = B.r[b] / h, d2 = sq_over(R, dn);
-  double fm[K2];
-  disk_square<Q>(cu, cv, d2 > 0.0 ? sqrt(d2) : 0.0, B.inside, S, fm);
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < K2; ++k) out[t * K2 + k] = fm[k];
-  }
+  const double fm = disk_square<Q, false>(cu, cv, d2 > 0.0 ? sqrt(d2) : 0.0, B.inside, S);
+  if (lane < K2) out[t * K2 + lane] = fm;
 }
 
 // a face next to a covered cell closes (3-D)
@@ -1711,18 +1839,28 @@ cudaError_t sphere_patch_launch(int q, const Spheres& B, const PatchRule& rule, 
   }
 }
 
-cudaError_t sphere_vol_launch(int q, const Spheres& B, const PatchRule& rule, int N, double h, const int32_t* cells,
-                              int64_t n, const int32_t* cbody, const double* volp, double* vol, cudaStream_t s) {
+template <int Q>
+cudaError_t vol_launch(const Spheres& B, const PatchRule& rule, const GlRuleT& glt, const GlRule& gl, int N, double h,
+                       const int32_t* cells, int64_t n, const int32_t* cbody, double* eb, double* ebn, double* volp, double* vol,
+                       cudaStream_t s) {
   const unsigned nb = (unsigned)((n + 3) / 4);
-  switch (q) {
-    case 0: k_sphere_vol<0><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol); break;
-    case 1: k_sphere_vol<1><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol); break;
-    case 2: k_sphere_vol<2><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol); break;
-    case 3: k_sphere_vol<3><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol); break;
-    default: k_sphere_vol<4><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol); break;
-  }
-  eb::count_launch();
+  k_sphere_vol<Q><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol, false);
+  k_sphere_patch_small<Q><<<(unsigned)n, SMALL_THREADS, 0, s>>>(B, glt, gl, N, h, cells, cbody, eb, ebn, volp, vol);
+  k_sphere_vol<Q><<<nb, 128, 0, s>>>(B, rule, N, h, cells, n, cbody, volp, vol, true);
+  eb::count_launches(3);
   return cudaGetLastError();
+}
+
+cudaError_t sphere_vol_launch(int q, const Spheres& B, const PatchRule& rule, const GlRuleT& glt, const GlRule& gl, int N,
+                              double h, const int32_t* cells, int64_t n, const int32_t* cbody, double* eb, double* ebn, double* volp,
+                              double* vol, cudaStream_t s) {
+  switch (q) {
+    case 0: return vol_launch<0>(B, rule, glt, gl, N, h, cells, n, cbody, eb, ebn, volp, vol, s);
+    case 1: return vol_launch<1>(B, rule, glt, gl, N, h, cells, n, cbody, eb, ebn, volp, vol, s);
+    case 2: return vol_launch<2>(B, rule, glt, gl, N, h, cells, n, cbody, eb, ebn, volp, vol, s);
+    case 3: return vol_launch<3>(B, rule, glt, gl, N, h, cells, n, cbody, eb, ebn, volp, vol, s);
+    default: return vol_launch<4>(B, rule, glt, gl, N, h, cells, n, cbody, eb, ebn, volp, vol, s);
+  }
 }
 
 cudaError_t sphere_faces_launch(int q, const Spheres& B, const PatchRule& rule, int N, int dir, double h,
@@ -1950,6 +2088,8 @@ extern "C" eb_status eb_geometry_spheres(int32_t N, int32_t n_body, const double
     if (!(B.r[b] > 0.0)) { set_error("eb_geometry_spheres: radii must be positive"); return EB_ERR_INVALID; }
   }
   static const PatchRule rule = patch_rule();
+  static const GlRuleT glt = gl_rule<GEO_GLT>();
+  static const GlRule gl = gl_rule<GEO_GL>();
   const double h = 1.0 / N;
   const int q = moment_degree, K = mono_count(3, q), KF = mono_count(2, q);
   cudaStream_t s = (cudaStream_t)stream;
@@ -2012,7 +2152,7 @@ extern "C" eb_status eb_geometry_spheres(int32_t N, int32_t n_body, const double
         if (nf0[d] > 0) GEO_TRY(sphere_faces_launch(q, B, rule, N, d, h, cf0[d], nf0[d], fbody[d], fm0[d], s));
       if (nc0 > 0) {
         GEO_TRY(sphere_patch_launch(q, B, rule, N, h, cut0, nc0, cbody, eb0, ebn0, volp, s));
-        GEO_TRY(sphere_vol_launch(q, B, rule, N, h, cut0, nc0, cbody, volp, vol0, s));
+        GEO_TRY(sphere_vol_launch(q, B, rule, glt, gl, N, h, cut0, nc0, cbody, eb0, ebn0, volp, vol0, s));
       }
       int32_t* keep;
       int64_t* pos;

@@ -1644,6 +1644,10 @@ static eb_status build_post(BuildCtx& c) {
     pl->tma32 = ok && (dm.n[0] % 4 == 0);
     pl->tma64 = ok && (dm.n[0] % 2 == 0);
     pl->seg = dm.nbr_box;
+    if (ok && D == 3 && pl->fsym && (R == 2 || R == 3)) {
+      EB_TRY(dalloc(st, &pl->fold_act, fold_act_size(pl->nx, pl->ny, pl->nz)));
+      EB_CUDA(fold_active(st->cell_kind, pl->nx, pl->ny, pl->nz, pl->fold_act, s));
+    }
     if (pl->seg && D == 3 && (R == 2 || R == 3) && st->n_irr > 0) EB_TRY(build_quad_plan(st, pl, R, s, tmp));
     EB_CUDA(cudaStreamCreateWithFlags(&pl->side, cudaStreamNonBlocking));
     EB_CUDA(cudaEventCreateWithFlags(&pl->fork, cudaEventDisableTiming));

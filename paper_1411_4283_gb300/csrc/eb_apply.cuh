@@ -69,11 +69,16 @@ struct ApplyPlan {
   int fsym = 0;                  // template even in x, y and z (to a few ulps): fully folded pass (3-D)
   std::vector<float> fold32;     // T(a, b, c), a, b, c in 0..R+1: the mean of the cube's eight sign images
   std::vector<double> fold64;
+  uint8_t* fold_act = nullptr;   // which groups of rows of the folded pass's tiles hold template cells (null: not used)
   int32_t* err;                  // device error word (bounded waits)
   cudaStream_t side;             // irregular pass runs here, overlapped with the template pass
   cudaEvent_t fork, join;
   int nsm;
 };
+
+// fold_act for the cell kinds (eb_apply_fold.cuh): its size and its values
+int64_t fold_act_size(int nx, int ny, int nz);
+cudaError_t fold_active(const uint8_t* kind, int nx, int ny, int nz, uint8_t* act, cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_apply(const ApplyArgs<T>& a, cudaStream_t s);

@@ -1084,7 +1084,7 @@ __host__ __device__ constexpr double half_pow(int sign, int e) {
 template <int Q>
 struct DiskSmem {
   double sn[GEO_GLT], cs[GEO_GLT], wt[GEO_GLT], br[4][8];
-  double node[4][32][Q + 3];  // weight, u, chord moments of v
+  double node[4][32][2 * Q + 3];  // weight times the powers of u, chord moments of v (odd: no bank conflicts)
 };
 template <int Q, bool CELL>
 __device__ __forceinline__ double disk_square(double cu, double cv, double rho, bool inside, DiskSmem<Q>& S) {
@@ -1124,14 +1124,15 @@ __device__ __forceinline__ double disk_square(double cu, double cv, double rho, 
         const double du = uq - cu, hw = sqrt(fmax(sq_less(rho, du), 0.0));
         const double va = fmin(fmax(cv - hw, -0.5), 0.5), vb = fmin(fmax(cv + hw, -0.5), 0.5);
         double* nd = S.node[warp][lane];
-        nd[0] = 0.5 * S.wt[i % GEO_GLT] * pw * M_PI * sn * S.cs[i % GEO_GLT];  // 0 on a panel of no width
-        nd[1] = uq;
-        double pa = va, pb = vb;
+        const double w = 0.5 * S.wt[i % GEO_GLT] * pw * M_PI * sn * S.cs[i % GEO_GLT];  // 0 on a panel of no width
+        double pa = va, pb = vb, up = 1.0;
 #pragma unroll
         for (int k = 0; k <= Q; ++k) {
           // the chord, or the two parts of the column beyond it
           const double full = half_pow(1, k + 1);
-          nd[2 + k] = inside ? (pb - pa) / (k + 1) : (pa - ((k & 1) ? full : -full)) / (k + 1) + (full - pb) / (k + 1);
+          nd[k] = w * up;
+          up *= uq;
+          nd[Q + 1 + k] = inside ? (pb - pa) / (k + 1) : (pa - ((k & 1) ? full : -full)) / (k + 1) + (full - pb) / (k + 1);
           pa = __dmul_rn(pa, va);  // not fused into the next difference
           pb = __dmul_rn(pb, vb);
         }
@@ -1141,9 +1142,7 @@ __device__ __forceinline__ double disk_square(double cu, double cv, double rho, 
       if (lane < K2)
         for (int j = 0; j < cnt; ++j) {
           const double* nd = S.node[warp][j];
-          double up = 1.0;
-          for (int e = 0; e < eu; ++e) up *= nd[1];
-          acc = fma(nd[0] * up, nd[2 + ev], acc);
+          acc = fma(nd[eu], nd[Q + 1 + ev], acc);
         }
       __syncwarp();
     }

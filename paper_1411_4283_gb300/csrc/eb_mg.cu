@@ -161,23 +161,31 @@ __global__ void k_mg_coarsen(int dim, int nxf, int nyf, int nzf, int nxc, int ny
   dgc[c] = -(cpl_sum + eb);
 }
 
-// y = M x on one level
-template <typename T>
-__device__ __forceinline__ T mg_apply_at(int dim, int nx, int ny, int nz, int64_t c, const int* x, const float* cp0,
-                                         const float* cp1, const float* cp2, const float* dg, const T* v) {
-  T s = (T)dg[c] * v[c];
+// sum of the couplings times the neighbours' values at cell c = p of a level; val(c, p) is a cell's value
+template <typename T, int D, typename Val>
+__device__ __forceinline__ T mg_offdiag(const int* n, int64_t c, const int* p, const float* cp0, const float* cp1,
+                                        const float* cp2, const Val& val) {
   const float* cp[3] = {cp0, cp1, cp2};
-  int64_t st[3] = {1, nx, (int64_t)nx * ny};
-  int n[3] = {nx, ny, nz};
-  for (int d = 0; d < dim; ++d) {
-    if (x[d] + 1 < n[d]) s += (T)cp[d][c] * v[c + st[d]];
-    if (x[d] > 0) s += (T)cp[d][c - st[d]] * v[c - st[d]];
+  const int64_t st[3] = {1, n[0], (int64_t)n[0] * n[1]};
+  T s = (T)0;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    int q[3] = {p[0], p[1], p[2]};
+    if (p[d] + 1 < n[d]) {
+      q[d] = p[d] + 1;
+      s += (T)__ldg(cp[d] + c) * val(c + st[d], q);
+    }
+    if (p[d] > 0) {
+      q[d] = p[d] - 1;
+      s += (T)__ldg(cp[d] + c - st[d]) * val(c - st[d], q);
+    }
   }
   return s;
 }
 
 // Level kernels run on a 3-D grid of (32 x 4)-thread blocks over (x, y) rows and z planes, so that a
-// thread's cell coordinates need no integer division.
+// thread's cell coordinates need no integer division.  The dimension is a template argument: with it at run time
+// the per-direction pointers and coordinates lived in local memory.
 constexpr int MG_BX = 32, MG_BY = 4;
 
 __device__ __forceinline__ bool mg_cell(int nx, int ny, int* p, int64_t* c) {
@@ -189,61 +197,86 @@ __device__ __forceinline__ bool mg_cell(int nx, int ny, int* p, int64_t* c) {
   return true;
 }
 
-// weighted Jacobi: out = x + w (b - M x) / diag   (x == null: out = w b / diag)
 template <typename T>
-__global__ void __launch_bounds__(MG_BX * MG_BY) k_mg_jacobi(int dim, int nx, int ny, int nz, const float* cp0,
-                                                             const float* cp1, const float* cp2, const float* dg,
-                                                             const T* __restrict__ b, const T* x, T* out, float w) {
+struct MgSweep {
+  int n[3], nc[2];        // cells of the level; of the coarser one in x and y (MG_POST)
+  const float* cp[3];
+  const float* dg;
+  const T* b;
+  const T* x;
+  const T* xc;            // the coarser level's correction (MG_POST)
+  T* out;
+  float w;
+};
+
+// Weighted Jacobi: out = x + w (b - M x) / diag.  A level's arrays mostly stay in L2 (128^3 in FP32: 14 us a sweep,
+// the loads of seven cells' values through L1), and on the coarser levels the launch bounds a pass, so there the
+// values that another pass would have written for the sweep are made on the fly:
+//   MG_FIRST, MG_PROLONG   no sweep: the first one from x = 0, out = w b / diag; x + x_c (piecewise constant on volumes)
+//   MG_PRE, MG_POST        those values and the sweep that follows, in one pass
+// The fused passes repeat a division or two more loads for each neighbour: 6.9 and 6.9 us at 64^3 in FP32 (two
+// passes: 8 and 9 us and a launch), but 29 and 30 us at 128^3 (20 and 24 us), hence the line between them; in FP64
+// the divide is a sequence on a pipe 64 times slower and the line lies lower.  The passes of a cycle at 128^3 took
+// 225 us in 18 launches before, 136 us in 14 now.
+enum { MG_PLAIN, MG_FIRST, MG_PROLONG, MG_PRE, MG_POST };
+template <typename T>
+constexpr int64_t MG_FUSE_CELLS = sizeof(T) == 4 ? 1 << 20 : 1 << 16;
+template <typename T, int D, int MODE>
+__global__ void __launch_bounds__(MG_BX * MG_BY) k_mg_jacobi(const __grid_constant__ MgSweep<T> a) {
   int p[3];
   int64_t c;
-  if (!mg_cell(nx, ny, p, &c)) return;
-  float d = dg[c];
-  if (d == 0.0f) { out[c] = (T)0; return; }
-  if (!x) { out[c] = (T)w * b[c] / (T)d; return; }
-  T r = b[c] - mg_apply_at<T>(dim, nx, ny, nz, c, p, cp0, cp1, cp2, dg, x);
-  out[c] = x[c] + (T)w * r / (T)d;
-}
-
-// coarse right-hand side: average of the children's residuals b - M x
-template <typename T>
-__global__ void __launch_bounds__(MG_BX * MG_BY) k_mg_restrict(int dim, int nxf, int nyf, int nzf, int nxc, int nyc, int nzc, const float* cp0,
-                              const float* cp1, const float* cp2, const float* dg, const T* __restrict__ b,
-                              const T* __restrict__ x, T* bc) {
-  int X[3];
-  int64_t c;
-  if (!mg_cell(nxc, nyc, X, &c)) return;
-  int nf[3] = {nxf, nyf, nzf};
-  const int nch = 1 << dim;
-  T acc = (T)0;
-  for (int k = 0; k < nch; ++k) {
-    int f[3] = {0, 0, 0};
-    bool in = true;
-    for (int d = 0; d < dim; ++d) {
-      f[d] = 2 * X[d] + ((k >> d) & 1);
-      if (f[d] >= nf[d]) in = false;
-    }
-    if (!in) continue;
-    int64_t fc = (int64_t)f[0] + (int64_t)nxf * ((int64_t)f[1] + (int64_t)nyf * f[2]);
-    if (dg[fc] == 0.0f) continue;
-    acc += b[fc] - mg_apply_at<T>(dim, nxf, nyf, nzf, fc, f, cp0, cp1, cp2, dg, x);
+  if (!mg_cell(a.n[0], a.n[1], p, &c)) return;
+  const float d = __ldg(a.dg + c);
+  if (d == 0.0f) {
+    a.out[c] = (T)0;
+    return;
   }
-  bc[c] = acc / (T)nch;
+  const auto val = [&](int64_t i, const int* q) -> T {
+    if (MODE == MG_PLAIN) return __ldg(a.x + i);
+    const float di = __ldg(a.dg + i);
+    if (MODE == MG_POST || MODE == MG_PROLONG) {
+      const T v = __ldg(a.x + i);
+      return di == 0.0f ? v : v + __ldg(a.xc + (q[0] >> 1) + (int64_t)a.nc[0] * ((q[1] >> 1) + (int64_t)a.nc[1] * (D == 3 ? q[2] >> 1 : 0)));
+    }
+    return di == 0.0f ? (T)0 : (T)a.w * __ldg(a.b + i) / (T)di;
+  };
+  const T v = val(c, p);
+  if (MODE == MG_FIRST || MODE == MG_PROLONG) {
+    a.out[c] = v;
+    return;
+  }
+  const T r = __ldg(a.b + c) - ((T)d * v + mg_offdiag<T, D>(a.n, c, p, a.cp[0], a.cp[1], a.cp[2], val));
+  a.out[c] = v + (T)a.w * r / (T)d;
 }
 
-// x_f += x_c (piecewise constant) on volumes
-template <typename T>
-__global__ void __launch_bounds__(MG_BX * MG_BY) k_mg_prolong(int dim, int nxf, int nyf, int nzf, int nxc, int nyc, const float* dg, const T* __restrict__ xc,
-                             T* xf) {
-  int p[3];
-  int64_t c;
-  if (!mg_cell(nxf, nyf, p, &c)) return;
-  if (dg[c] == 0.0f) return;
-  int64_t cc = (int64_t)(p[0] >> 1) + (int64_t)nxc * ((int64_t)(p[1] >> 1) + (int64_t)nyc * (dim == 3 ? (p[2] >> 1) : 0));
-  xf[c] += xc[cc];
+// coarse right-hand side: average of the children's residuals b - M x.  A lane takes the children of one fine x (two
+// or four, a warp thereby reads whole rows) and adds its neighbour's: with a thread per coarse cell the chain of its
+// eight children's loads was the time on the coarser levels (10 us from 32^3 cells and 20 us from 128^3, 9 and 16 us now).
+template <typename T, int D>
+__global__ void __launch_bounds__(MG_BX * MG_BY) k_mg_restrict(const __grid_constant__ MgSweep<T> a) {
+  const int fx = blockIdx.x * MG_BX + threadIdx.x, Y = blockIdx.y * MG_BY + threadIdx.y, Z = blockIdx.z;
+  if (Y >= a.nc[1]) return;  // a whole warp
+  const auto val = [&](int64_t i, const int*) { return __ldg(a.x + i); };
+  T acc = (T)0;
+#pragma unroll
+  for (int k = 0; k < (1 << (D - 1)); ++k) {
+    const int f[3] = {fx, 2 * Y + (k & 1), D == 3 ? 2 * Z + (k >> 1) : 0};
+    if (f[0] >= a.n[0] || f[1] >= a.n[1] || (D == 3 && f[2] >= a.n[2])) continue;
+    const int64_t fc = (int64_t)f[0] + (int64_t)a.n[0] * ((int64_t)f[1] + (int64_t)a.n[1] * f[2]);
+    const float d = __ldg(a.dg + fc);
+    if (d == 0.0f) continue;
+    acc += __ldg(a.b + fc) - ((T)d * __ldg(a.x + fc) + mg_offdiag<T, D>(a.n, fc, f, a.cp[0], a.cp[1], a.cp[2], val));
+  }
+  acc += __shfl_down_sync(0xffffffffu, acc, 1);
+  if (!(fx & 1) && fx < a.n[0])
+    a.out[(fx >> 1) + (int64_t)a.nc[0] * ((int64_t)Y + (int64_t)a.nc[1] * Z)] = acc / (T)(1 << D);
 }
 
-// The levels from `l0` down, when small, in one CTA: the same V-cycle with
-// block-wide barriers instead of kernel boundaries.
+// The levels from `l0` down, when small, in one CTA: the same V-cycle with block-wide barriers instead of kernel
+// boundaries.  What bounds it is the latency of some forty dependent phases, so all levels lie in shared memory:
+// right-hand side, iterate and its copy, w / diag, couplings, which neighbours exist and the parent's index; a
+// level's phases are run by as many warps as it has cells for.  From global memory a phase took 2 us (16^3 in FP32:
+// 85 us a cycle, 33 now).
 template <typename T>
 struct MgDev {
   int n[3];
@@ -253,90 +286,141 @@ struct MgDev {
   T* x;
   T* w;
 };
-
-template <typename T>
-__device__ void cta_jacobi(int dim, const MgDev<T>& L, const T* x, T* out, float om) {
-  int64_t n = (int64_t)L.n[0] * L.n[1] * L.n[2];
-  for (int64_t c = threadIdx.x; c < n; c += blockDim.x) {
-    float d = L.dg[c];
-    if (d == 0.0f) { out[c] = (T)0; continue; }
-    if (!x) { out[c] = (T)om * L.b[c] / (T)d; continue; }
-    int p[3];
-    xyz_of(c, L.n[0], L.n[1], p);
-    T r = L.b[c] - mg_apply_at<T>(dim, L.n[0], L.n[1], L.n[2], c, p, L.cp[0], L.cp[1], L.cp[2], L.dg, x);
-    out[c] = x[c] + (T)om * r / (T)d;
-  }
+constexpr int MG_CTA_THREADS = 1024;
+template <typename T, int D>
+__host__ __device__ constexpr int64_t mg_cta_bytes(int64_t cells) {  // of one level (16-byte multiple)
+  return (cells * (4 * (int64_t)sizeof(T) + 4 * D + 3) + 15) / 16 * 16;
 }
-
-template <typename T>
-__global__ void __launch_bounds__(1024) k_mg_coarse(int dim, int nlev, const MgDev<T>* __restrict__ lev, float om,
-                                                    int nu, int ncoarse) {
-  // per-thread copies of the ping-pong pointers (identical in every thread)
-  T* xs[MG_MAXLEV];
-  T* ws[MG_MAXLEV];
-  for (int l = 0; l < nlev; ++l) {
-    xs[l] = lev[l].x;
-    ws[l] = lev[l].w;
+template <typename T, int D>
+struct MgShared {
+  int n[3], cells, threads;
+  T *b, *x, *w, *id;
+  float* cp;        // [D][cells]
+  uint16_t* parent;
+  uint8_t* nb;      // bit 2 d: a neighbour above in direction d, bit 2 d + 1: below
+  __device__ MgShared(const MgDev<T>& L, unsigned char* at) {
+    for (int d = 0; d < 3; ++d) n[d] = L.n[d];
+    cells = n[0] * n[1] * n[2];
+    threads = min(MG_CTA_THREADS, (cells + 31) / 32 * 32);
+    b = reinterpret_cast<T*>(at);
+    x = b + cells;
+    w = x + cells;
+    id = w + cells;
+    cp = reinterpret_cast<float*>(id + cells);
+    parent = reinterpret_cast<uint16_t*>(cp + D * cells);
+    nb = reinterpret_cast<uint8_t*>(parent + cells);
   }
-  for (int l = 0; l < nlev; ++l) {  // descend
-    MgDev<T> L = lev[l];
-    const bool last = l == nlev - 1;
-    const int sweeps = last ? ncoarse : nu;
-    cta_jacobi<T>(dim, L, nullptr, xs[l], om);
-    __syncthreads();
-    for (int it = 1; it < sweeps; ++it) {
-      cta_jacobi<T>(dim, L, xs[l], ws[l], om);
-      __syncthreads();
-      T* t = xs[l]; xs[l] = ws[l]; ws[l] = t;
+  __device__ __forceinline__ T offdiag(int c, const T* v) const {
+    const int m = nb[c], st[3] = {1, n[0], n[0] * n[1]};
+    T s = (T)0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      if (m >> (2 * d) & 1) s += (T)cp[d * cells + c] * v[c + st[d]];
+      if (m >> (2 * d + 1) & 1) s += (T)cp[d * cells + c - st[d]] * v[c - st[d]];
     }
-    if (!last) {
-      MgDev<T> C = lev[l + 1];
-      int64_t ncc = (int64_t)C.n[0] * C.n[1] * C.n[2];
-      const int nch = 1 << dim;
-      for (int64_t c = threadIdx.x; c < ncc; c += blockDim.x) {
-        int X[3];
-        xyz_of(c, C.n[0], C.n[1], X);
-        T acc = (T)0;
-        for (int k = 0; k < nch; ++k) {
-          int f[3] = {0, 0, 0};
-          bool in = true;
-          for (int d = 0; d < dim; ++d) {
-            f[d] = 2 * X[d] + ((k >> d) & 1);
-            if (f[d] >= L.n[d]) in = false;
-          }
-          if (!in) continue;
-          int64_t fc = (int64_t)f[0] + (int64_t)L.n[0] * ((int64_t)f[1] + (int64_t)L.n[1] * f[2]);
-          if (L.dg[fc] == 0.0f) continue;
-          acc += L.b[fc] - mg_apply_at<T>(dim, L.n[0], L.n[1], L.n[2], fc, f, L.cp[0], L.cp[1], L.cp[2], L.dg, xs[l]);
-        }
-        C.b[c] = acc / (T)nch;
+    return s;
+  }
+  __device__ __forceinline__ void sync() const {  // the level's warps
+    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+  }
+  // x + w (b - M x) / diag = (1 - w) x + (w / diag) (b - couplings)
+  __device__ void sweeps(int count, float om) {
+    for (int it = 0; it < count; ++it) {
+      for (int c = threadIdx.x; c < cells; c += threads)
+        w[c] = id[c] == (T)0 ? (T)0 : ((T)1 - (T)om) * x[c] + id[c] * (b[c] - offdiag(c, x));
+      sync();
+      T* t = x;
+      x = w;
+      w = t;
+    }
+  }
+};
+
+template <typename T, int D>
+__global__ void __launch_bounds__(MG_CTA_THREADS) k_mg_coarse(int nlev, const MgDev<T>* __restrict__ lev, float om, int nu,
+                                                              int ncoarse) {
+  extern __shared__ __align__(16) unsigned char mg_smem[];
+  const int tid = threadIdx.x;
+  int64_t at = 0;
+  for (int l = 0; l < nlev; ++l) {
+    const MgDev<T> L = lev[l];
+    const MgShared<T, D> S(L, mg_smem + at);
+    at += mg_cta_bytes<T, D>(S.cells);
+    const int mx = (S.n[0] + 1) / 2, my = (S.n[1] + 1) / 2;
+    for (int c = tid; c < S.cells; c += MG_CTA_THREADS) {
+      const float d = L.dg[c];
+      S.id[c] = d == 0.0f ? (T)0 : (T)om / (T)d;
+      if (l == 0) S.b[c] = L.b[c];
+      const int p[3] = {c % S.n[0], c / S.n[0] % S.n[1], c / (S.n[0] * S.n[1])};
+      int m = 0;
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        S.cp[k * S.cells + c] = L.cp[k][c];
+        m |= (p[k] + 1 < S.n[k]) << (2 * k) | (p[k] > 0) << (2 * k + 1);
       }
-      __syncthreads();
+      S.nb[c] = (uint8_t)m;
+      S.parent[c] = (uint16_t)((p[0] >> 1) + mx * ((p[1] >> 1) + my * (D == 3 ? p[2] >> 1 : 0)));
     }
+  }
+  __syncthreads();
+  // descend; odd sweep counts leave a level's iterate in its other buffer (bit l of odd)
+  unsigned odd = 0;
+  at = 0;
+  for (int l = 0; l < nlev; ++l) {
+    MgShared<T, D> S(lev[l], mg_smem + at);
+    const int64_t here = at;
+    at += mg_cta_bytes<T, D>(S.cells);
+    const bool last = l == nlev - 1;
+    const int more = (last ? ncoarse : nu) - 1;
+    if (tid < S.threads) {
+      for (int c = tid; c < S.cells; c += S.threads) S.x[c] = S.id[c] * S.b[c];
+      S.sync();
+      S.sweeps(more, om);
+    }
+    odd |= (unsigned)(more & 1) << l;
+    __syncthreads();
+    if (last) break;
+    const MgShared<T, D> F(lev[l], mg_smem + here), C(lev[l + 1], mg_smem + at);
+    const T* x = (more & 1) ? F.w : F.x;
+    const float* dg = lev[l].dg;
+    for (int c = tid; c < C.cells; c += MG_CTA_THREADS) {
+      const int X[3] = {c % C.n[0], c / C.n[0] % C.n[1], c / (C.n[0] * C.n[1])};
+      T acc = (T)0;
+#pragma unroll
+      for (int k = 0; k < (1 << D); ++k) {
+        const int f0 = 2 * X[0] + (k & 1), f1 = 2 * X[1] + ((k >> 1) & 1), f2 = D == 3 ? 2 * X[2] + (k >> 2) : 0;
+        if (f0 >= F.n[0] || f1 >= F.n[1] || (D == 3 && f2 >= F.n[2])) continue;
+        const int fc = f0 + F.n[0] * (f1 + F.n[1] * f2);
+        const float d = __ldg(dg + fc);
+        if (d != 0.0f) acc += F.b[fc] - ((T)d * x[fc] + F.offdiag(fc, x));
+      }
+      C.b[c] = acc / (T)(1 << D);
+    }
+    __syncthreads();
   }
   for (int l = nlev - 2; l >= 0; --l) {  // ascend
-    MgDev<T> L = lev[l];
-    MgDev<T> C = lev[l + 1];
-    int64_t n = (int64_t)L.n[0] * L.n[1] * L.n[2];
-    for (int64_t c = threadIdx.x; c < n; c += blockDim.x) {
-      if (L.dg[c] == 0.0f) continue;
-      int p[3];
-      xyz_of(c, L.n[0], L.n[1], p);
-      int64_t cc = (int64_t)(p[0] >> 1) + (int64_t)C.n[0] * ((int64_t)(p[1] >> 1) + (int64_t)C.n[1] * (dim == 3 ? (p[2] >> 1) : 0));
-      xs[l][c] += xs[l + 1][cc];
+    at = 0;
+    for (int k = 0; k < l; ++k) at += mg_cta_bytes<T, D>((int64_t)lev[k].n[0] * lev[k].n[1] * lev[k].n[2]);
+    MgShared<T, D> S(lev[l], mg_smem + at);
+    const MgShared<T, D> C(lev[l + 1], mg_smem + at + mg_cta_bytes<T, D>(S.cells));
+    const T* xc = (odd >> (l + 1) & 1) ? C.w : C.x;
+    if (odd >> l & 1) {
+      T* t = S.x;
+      S.x = S.w;
+      S.w = t;
     }
+    if (tid < S.threads) {
+      for (int c = tid; c < S.cells; c += S.threads)
+        if (S.id[c] != (T)0) S.x[c] += xc[S.parent[c]];
+      S.sync();
+      S.sweeps(nu, om);
+    }
+    odd ^= (unsigned)(nu & 1) << l;
     __syncthreads();
-    for (int it = 0; it < nu; ++it) {
-      cta_jacobi<T>(dim, L, xs[l], ws[l], om);
-      __syncthreads();
-      T* t = xs[l]; xs[l] = ws[l]; ws[l] = t;
-    }
   }
-  // the group's result belongs in level 0's x buffer
-  if (xs[0] != lev[0].x) {
-    int64_t n = (int64_t)lev[0].n[0] * lev[0].n[1] * lev[0].n[2];
-    for (int64_t c = threadIdx.x; c < n; c += blockDim.x) lev[0].x[c] = xs[0][c];
-  }
+  const MgShared<T, D> S(lev[0], mg_smem);
+  const T* x = (odd & 1) ? S.w : S.x;
+  for (int c = tid; c < S.cells; c += MG_CTA_THREADS) lev[0].x[c] = x[c];
 }
 
 static unsigned nb256(int64_t n) { return (unsigned)((n + 255) / 256); }
@@ -615,6 +699,15 @@ static cudaError_t blocks_setup(const MgFineInput& in, Multigrid* mg, const int3
   return cudaGetLastError();
 }
 
+static cudaError_t mg_cta_attributes() {
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const int bytes = 227 * 1024;
+  cudaError_t e = cudaFuncSetAttribute(k_mg_coarse<float, 2>, attr, bytes);
+  if (!e) e = cudaFuncSetAttribute(k_mg_coarse<float, 3>, attr, bytes);
+  if (!e) e = cudaFuncSetAttribute(k_mg_coarse<double, 2>, attr, bytes);
+  return e ? e : cudaFuncSetAttribute(k_mg_coarse<double, 3>, attr, bytes);
+}
+
 cudaError_t mg_setup(const MgFineInput& in, Multigrid* mg, cudaStream_t s) {
   mg->dim = in.dim;
   mg->nlev = 0;
@@ -671,6 +764,7 @@ cudaError_t mg_setup(const MgFineInput& in, Multigrid* mg, cudaStream_t s) {
     h32[l].b = L.v32[0]; h32[l].x = L.v32[1]; h32[l].w = L.v32[2];
     h64[l].b = L.v64[0]; h64[l].x = L.v64[1]; h64[l].w = L.v64[2];
   }
+  if ((e = mg_cta_attributes())) return e;
   if ((e = cudaMalloc(&mg->dev32, sizeof(h32)))) return e;
   if ((e = cudaMalloc(&mg->dev64, sizeof(h64)))) return e;
   if ((e = cudaMemcpyAsync(mg->dev32, h32, sizeof(h32), cudaMemcpyHostToDevice, s))) return e;
@@ -715,59 +809,93 @@ template <>
 double* vbuf<double>(MgLevel& L, int k) { return L.v64[k]; }
 
 // z = V(b) on level l; b and z live in the level's buffers (0: b, 1: x, 2: work)
-constexpr int64_t MG_CTA_CELLS = 4096;  // levels at most this large run inside one CTA
+constexpr int64_t MG_CTA_CELLS = 4096;            // levels at most this large run inside one CTA ...
+constexpr int64_t MG_CTA_SMEM = 227 * 1024;       // ... if they and the coarser ones fit its shared memory
+
+// shared memory of the levels from l down (MG_CTA_SMEM + 1: not in one CTA)
+template <typename T, int D>
+static int64_t mg_cta_smem(const Multigrid& mg, int l) {
+  if (mg.lev[l].ncell > MG_CTA_CELLS) return MG_CTA_SMEM + 1;
+  int64_t bytes = 0;
+  for (int k = l; k < mg.nlev; ++k) bytes += mg_cta_bytes<T, D>(mg.lev[k].ncell);
+  return bytes;
+}
 
 static dim3 mg_grid(const int* n) {
   return dim3((unsigned)((n[0] + MG_BX - 1) / MG_BX), (unsigned)((n[1] + MG_BY - 1) / MG_BY), (unsigned)n[2]);
 }
 
-template <typename T>
+template <typename T, int D>
 static cudaError_t vcycle(const Multigrid& mgc, int l, cudaStream_t s) {
   Multigrid& mg = const_cast<Multigrid&>(mgc);
   MgLevel& L = mg.lev[l];
-  if (L.ncell <= MG_CTA_CELLS) {
-    const int D = mg.dim;
+  const float om = 0.8f;
+  const int64_t smem = mg_cta_smem<T, D>(mg, l);
+  if (smem <= MG_CTA_SMEM) {
     MgDev<T>* dev = sizeof(T) == 4 ? (MgDev<T>*)mg.dev32 : (MgDev<T>*)mg.dev64;
-    k_mg_coarse<T><<<1, 1024, 0, s>>>(D, mg.nlev - l, dev + l, 0.8f, MG_NU, 24);
+    k_mg_coarse<T, D><<<1, MG_CTA_THREADS, smem, s>>>(mg.nlev - l, dev + l, om, MG_NU, 24);
     eb::count_launch();
     return cudaGetLastError();
   }
-  T* b = vbuf<T>(L, 0);
-  const int D = mg.dim;
-  const float om = 0.8f;
+  static_assert(MG_NU >= 2, "MG_PRE makes two sweeps");
   const bool coarsest = l == mg.nlev - 1;
-  const int pre = coarsest ? 24 : MG_NU;
-  const int post = coarsest ? 0 : MG_NU;
-  // the level's result ends in buffer 1: the first smoothing step writes buffer 1 or 2 by the parity
-  // of the sweeps that follow it
-  T* x = vbuf<T>(L, (pre - 1 + post) % 2 == 0 ? 1 : 2);
-  T* w = vbuf<T>(L, (pre - 1 + post) % 2 == 0 ? 2 : 1);
+  const int pre = coarsest ? 24 : MG_NU, post = coarsest ? 0 : MG_NU;
+  const bool fuse = L.ncell <= MG_FUSE_CELLS<T>;
+  const int first = fuse ? 2 : 1;  // sweeps of the first kernel
+  // the level's result ends in buffer 1: the first kernel writes buffer 1 or 2 by the parity of the passes that
+  // follow it
+  const bool even = (pre - first + post + (coarsest || fuse ? 0 : 1)) % 2 == 0;
+  T* x = vbuf<T>(L, even ? 1 : 2);
+  T* w = vbuf<T>(L, even ? 2 : 1);
   const dim3 blk(MG_BX, MG_BY), grd = mg_grid(L.n);
-  // smoothing: x = w b / d, then sweeps ping-ponging x <-> w
-  k_mg_jacobi<T><<<grd, blk, 0, s>>>(D, L.n[0], L.n[1], L.n[2], L.cp[0], L.cp[1], L.cp[2], L.dg, b, nullptr, x, om);
-  eb::count_launch();
-  for (int it = 1; it < pre; ++it) {
-    k_mg_jacobi<T><<<grd, blk, 0, s>>>(D, L.n[0], L.n[1], L.n[2], L.cp[0], L.cp[1], L.cp[2], L.dg, b, x, w, om);
-    eb::count_launch();
-    T* t = x; x = w; w = t;
+  MgSweep<T> a;
+  for (int d = 0; d < 3; ++d) {
+    a.n[d] = L.n[d];
+    a.cp[d] = L.cp[d];
   }
+  a.nc[0] = a.nc[1] = 0;
+  a.dg = L.dg;
+  a.b = vbuf<T>(L, 0);
+  a.x = a.xc = nullptr;
+  a.out = x;
+  a.w = om;
+  if (fuse) k_mg_jacobi<T, D, MG_PRE><<<grd, blk, 0, s>>>(a);
+  else k_mg_jacobi<T, D, MG_FIRST><<<grd, blk, 0, s>>>(a);
+  eb::count_launch();
+  const auto pass = [&](int mode) {
+    a.x = x;
+    a.out = w;
+    if (mode == MG_POST) k_mg_jacobi<T, D, MG_POST><<<grd, blk, 0, s>>>(a);
+    else if (mode == MG_PROLONG) k_mg_jacobi<T, D, MG_PROLONG><<<grd, blk, 0, s>>>(a);
+    else k_mg_jacobi<T, D, MG_PLAIN><<<grd, blk, 0, s>>>(a);
+    eb::count_launch();
+    T* t = x;
+    x = w;
+    w = t;
+  };
+  for (int it = first; it < pre; ++it) pass(MG_PLAIN);
   if (!coarsest) {
     MgLevel& C = mg.lev[l + 1];
-    k_mg_restrict<T><<<mg_grid(C.n), blk, 0, s>>>(D, L.n[0], L.n[1], L.n[2], C.n[0], C.n[1], C.n[2], L.cp[0], L.cp[1],
-                                                 L.cp[2], L.dg, b, x, vbuf<T>(C, 0));
+    a.nc[0] = C.n[0];
+    a.nc[1] = C.n[1];
+    a.x = x;
+    a.out = vbuf<T>(C, 0);
+    const int rows[3] = {L.n[0], C.n[1], C.n[2]};
+    k_mg_restrict<T, D><<<mg_grid(rows), blk, 0, s>>>(a);
     eb::count_launch();
-    cudaError_t e = vcycle<T>(mg, l + 1, s);
+    const cudaError_t e = vcycle<T, D>(mg, l + 1, s);
     if (e) return e;
-    k_mg_prolong<T><<<grd, blk, 0, s>>>(D, L.n[0], L.n[1], L.n[2], C.n[0], C.n[1], L.dg, vbuf<T>(C, 1), x);
-    eb::count_launch();
-    for (int it = 0; it < post; ++it) {
-      k_mg_jacobi<T><<<grd, blk, 0, s>>>(D, L.n[0], L.n[1], L.n[2], L.cp[0], L.cp[1], L.cp[2], L.dg, b, x, w, om);
-      eb::count_launch();
-      T* t = x; x = w; w = t;
-    }
+    a.xc = vbuf<T>(C, 1);
+    pass(fuse ? MG_POST : MG_PROLONG);
+    for (int it = fuse ? 1 : 0; it < post; ++it) pass(MG_PLAIN);
   }
   if (x != vbuf<T>(L, 1)) return cudaErrorUnknown;  // parity bookkeeping above
   return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t vcycle(const Multigrid& mg, cudaStream_t s) {
+  return mg.dim == 3 ? vcycle<T, 3>(mg, 0, s) : vcycle<T, 2>(mg, 0, s);
 }
 
 // The V-cycle works on the levels' fixed buffers, so it is captured once per
@@ -787,7 +915,7 @@ cudaError_t mg_precond(const Multigrid& mgc, const T* r, T* z, cudaStream_t s) {
     if ((e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking))) return e;
     long long before = eb::launches_so_far();
     if ((e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal))) { cudaStreamDestroy(cap); return e; }
-    cudaError_t ev = vcycle<T>(mg, 0, cap);
+    cudaError_t ev = vcycle<T>(mg, cap);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(cap, &graph);
     cudaStreamDestroy(cap);
@@ -801,7 +929,7 @@ cudaError_t mg_precond(const Multigrid& mgc, const T* r, T* z, cudaStream_t s) {
   }
   if ((e = cudaMemcpyAsync(vbuf<T>(L, 0), r, L.ncell * sizeof(T), cudaMemcpyDeviceToDevice, s))) return e;
   if (capturing) {
-    if ((e = vcycle<T>(mg, 0, s))) return e;
+    if ((e = vcycle<T>(mg, s))) return e;
   } else {
     if ((e = cudaGraphLaunch(mg.exec[k], s))) return e;
     eb::count_launches(mg.nodes[k]);

@@ -44,10 +44,9 @@ sys.path.insert(0, ROOT)
 
 METRIC = "cut-face LS stencils/s; EB Laplacian apply GB/s (% HBM); solve s at fixed error"
 # DRAM bytes (read + write) of the least-squares launch per LS system solved, from an ncu capture of
-# the 48^3 sphere build (the mixed path, k_lsq<false, float>): 9.848 GB read + 16.650 GB written for
-# 90,123 systems.  The traffic is the per-system scratch (FP64 rows staged, then read by every
-# correction) of the ~900 systems in flight, which exceeds L2.
-LSQ_DRAM_BYTES_PER_SYSTEM = (9.848110e9 + 16.649961e9) / 90123
+# the 48^3 sphere build (k_lsq_mixed): 0.195 GB read + 0.508 GB written for 90,123 systems: the moment
+# tables and the stencils (the rows of a system lie in registers).
+LSQ_DRAM_BYTES_PER_SYSTEM = (0.195361e9 + 0.507776e9) / 90123
 
 
 def parse():
@@ -482,12 +481,12 @@ def main():
     lsq_share = lsq_ms / ms_step
     if lsq_share >= apply_share:
         # DRAM traffic of k_lsq: ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch on the 48^3
-        # sphere workload (8.19 GB for 90,123 systems), scaled by the systems of this launch
+        # sphere workload (0.70 GB for 90,123 systems), scaled by the systems of this launch
         traffic = LSQ_DRAM_BYTES_PER_SYSTEM * n_solved if args.order == 4 else None
         ex64 = bi["ls_fp64_flops"] / (lsq_ms / 1e3) / 1e12
         ex32 = bi["ls_fp32_flops"] / (lsq_ms / 1e3) / 1e12
-        roof = {"kernel": "k_lsq (weighted least squares: FP32 Householder factor, FP64 corrected semi-normal "
-                          "iterations; FP64 Householder for the systems the FP32 factor leaves)",
+        roof = {"kernel": "k_lsq_mixed (weighted least squares: FP32 Gram-Schmidt factor, FP64 passes and compensated "
+                          "FP32 corrections; FP64 Householder for the systems the FP32 factor leaves)",
                 "bound": "alu", "achieved": lsq_tflops,
                 "peak": fp64_pk, "unit": "TFLOP/s", "frac": lsq_tflops / fp64_pk, "traffic": traffic,
                 "achieved_note": "the method's FP64 Householder flop count (2nK^2 - 2K^3/3 + 4nK + K^2 per system "

@@ -102,8 +102,8 @@ typedef struct eb_params {
   double w_threshold;    /* 0.5 */
   double w_power;        /* 5 */
   int32_t ls_precision;  /* EB_LS_MIXED (default): each least-squares system is factorised in FP32
-                            and solved by FP64 corrected semi-normal iterations preconditioned by that
-                            factor, a system the FP32 factor cannot carry going to the FP64 path;
+                            and solved by corrected semi-normal iterations preconditioned by that factor
+                            (FP64 passes and compensated FP32 corrections), a system the FP32 factor cannot carry going to the FP64 path;
                             EB_LS_FP64: FP64 Householder factorisation for every system.  Both give
                             the FP64 minimum-norm stencil to rounding (Sec. 2.2.1). */
 } eb_params;

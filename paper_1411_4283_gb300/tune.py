@@ -1,10 +1,10 @@
 """Autotuner of the compile-time kernel shapes, run on the target GPU.
 
-The least-squares kernel's shape is fixed at compile time: how many systems one CTA keeps in
-flight (EB_LS_SYS_F for the FP32-factorisation kernel, the default path; EB_LS_SYS for the FP64
-one; their shared-memory blocks must fit in 227 KB) and how many rows each lane holds per chunk
-(EB_LS_RPL, shared by both; larger chunks amortise the per-step Householder scalars and column sums
-over more rows but leave fewer warps per SM to hide the serial parts).  Each candidate is compiled
+The least-squares kernels' shapes are fixed at compile time: for the FP32-factorisation kernel, the
+default path, how many warps the CTA of one system has (EB_LS_W) and how many such CTAs an SM keeps
+(EB_LS_CTAS: the rows lie in registers, so more CTAs mean fewer registers a thread); for the FP64 kernel,
+how many systems one CTA keeps in flight (EB_LS_SYS; their shared-memory blocks must fit in 227 KB) and
+how many rows each lane holds per chunk (EB_LS_RPL).  Each candidate is compiled
 into its own copy of the library (a candidate whose blocks do not fit fails its compile-time check
 and is skipped), timed in a fresh process that builds the stencils of the 3-D sphere workload and
 reads the least-squares launches' device time, and the fastest (the built-in default unless another
@@ -34,14 +34,12 @@ from . import build as _build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
-# candidate shapes: the defines of each (FP32 systems per CTA, rows per lane, FP64 systems per CTA)
+# candidate shapes: the defines of each (FP32 kernel: warps per system, CTAs per SM; FP64 kernel: systems per CTA,
+# rows per lane)
 CANDIDATES = [
-    {"EB_LS_SYS_F": 6, "EB_LS_RPL": 4, "EB_LS_SYS": 4},  # the built-in default: kept unless beaten by MARGIN
-    {"EB_LS_SYS_F": 7, "EB_LS_RPL": 4, "EB_LS_SYS": 4},
-    {"EB_LS_SYS_F": 5, "EB_LS_RPL": 4, "EB_LS_SYS": 4},
-    {"EB_LS_SYS_F": 4, "EB_LS_RPL": 4, "EB_LS_SYS": 4},
-    {"EB_LS_SYS_F": 4, "EB_LS_RPL": 6, "EB_LS_SYS": 3},
-    {"EB_LS_SYS_F": 3, "EB_LS_RPL": 8, "EB_LS_SYS": 2},
+    {"EB_LS_W": 4, "EB_LS_CTAS": 2, "EB_LS_SYS": 4, "EB_LS_RPL": 4},  # the built-in default: kept unless beaten by MARGIN
+    {"EB_LS_W": 4, "EB_LS_CTAS": 3, "EB_LS_SYS": 4, "EB_LS_RPL": 4},
+    {"EB_LS_W": 7, "EB_LS_CTAS": 2, "EB_LS_SYS": 4, "EB_LS_RPL": 4},
 ]
 
 

@@ -532,11 +532,16 @@ cudaError_t launch_apply(const ApplyArgs<T>& a, cudaStream_t s) {
     if ((e = launch_irregular<T>(a, fork ? pl->side : s))) return e;
   }
   if (a.n_irr > 0 && use_runs(a)) {
-    // the wall-layer class cells (FMA-bound, rows L2-resident) follow the template pass on the main
-    // stream while the HBM-bound unique-row stream runs on the side stream
+    // The wall-layer class cells (FMA-bound, rows L2-resident) follow the template pass on the main stream while the
+    // HBM-bound unique-row stream runs on the side stream.  In FP64 all but that stream is bound by the FP64 pipe,
+    // and each pass alone leaves it idle in its last wave and its barriers: the slab bricks and the rest go behind
+    // the row stream, beside the template pass (750 -> 496 us at 64^3, 2640 -> 2296 us at 160^3, 5809 -> 5168 us at
+    // 220^3).  In FP32 the row stream is the longer side already: the same move takes 164 -> 202 us at 128^3 and gains
+    // 1 % at 256^3, the runs alone 164 -> 176 us and 2 %.
+    const cudaStream_t wall = sizeof(T) == 8 && fork ? pl->side : s;
     if ((e = launch_runs<T>(a, s))) return e;
-    if (pl->brick && (e = launch_brick<T>(a, s))) return e;
-    if (pl->nL > 0 && (e = launch_seg_rest<T>(a, s))) return e;
+    if (pl->brick && (e = launch_brick<T>(a, wall))) return e;
+    if (pl->nL > 0 && (e = launch_seg_rest<T>(a, wall))) return e;
   }
   if (fork) {
     if ((e = cudaEventRecord(pl->join, pl->side))) return e;

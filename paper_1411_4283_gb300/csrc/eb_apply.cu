@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(256) k_apply_irregular(ApplyArgs<T> a) {
 // 100^3 grid take 56 us in FP32, and 17 us with W = 8 (FP64 at 160^3, 50000
 // rows: 131 and 55 us).  From SEG_MANY rows on, where there are warps enough,
 // the repeated index work costs more than it gives (FP32, 280000 rows: 91 and
-// 93 us; 930000 rows: 306 and 370 us).
+// 93 us; 1.15 M rows: 306 and 370 us).
 constexpr int SEG_BLOCK_WARPS = 8;
 constexpr int64_t SEG_MANY = 262144;
 

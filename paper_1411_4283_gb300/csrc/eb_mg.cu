@@ -214,8 +214,8 @@ struct MgSweep {
 // values that another pass would have written for the sweep are made on the fly:
 //   MG_FIRST, MG_PROLONG   no sweep: the first one from x = 0, out = w b / diag; x + x_c (piecewise constant on volumes)
 //   MG_PRE, MG_POST        those values and the sweep that follows, in one pass
-// The fused passes repeat a division or two more loads for each neighbour: 6.9 and 6.9 us at 64^3 in FP32 (two
-// passes: 8 and 9 us and a launch), but 29 and 30 us at 128^3 (20 and 24 us), hence the line between them; in FP64
+// The fused passes repeat a division or two more loads for each neighbour: 6.9 and 7.1 us at 64^3 in FP32 (4.8
+// for the sweep alone, before another pass and its launch), but 29 and 30 us at 128^3 (two passes: 25 and 26 us), hence the line between them; in FP64
 // the divide is a sequence on a pipe 64 times slower and the line lies lower.  The passes of a cycle at 128^3 took
 // 225 us in 18 launches before, 136 us in 14 now.
 enum { MG_PLAIN, MG_FIRST, MG_PROLONG, MG_PRE, MG_POST };

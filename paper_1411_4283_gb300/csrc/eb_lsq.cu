@@ -193,7 +193,7 @@ struct __align__(16) MixSmem {
   int32_t cnt[W][2];
   uint16_t orig[NR];    // its place in the row list
   int32_t slot;
-  float norm0;
+  double down;          // undoes the scale of F
 };
 
 template <int K, int W, int R>
@@ -529,10 +529,26 @@ __global__ void __launch_bounds__(W > 1 ? 32 * W : 128, MINB)
           f = (double)T.mon[i][dface] * mq;
         }
       }
-      S.F[i] = f;
-      S.rf[i] = (float)f;
+      S.r[i] = f;
     }
     group_sync<W>();
+    // F scaled to size one by a power of two, which passes every rounding, so that the coefficients scale with the
+    // face's moments: the solves' FP32 numbers, and the squares in the size of a correction, do not hold every scale
+    // (F at 1e-18: the corrections' squares were zero, the system passed for settled and t was 1e-8 off; at 1e21
+    // their overflow did the same).  F that is zero, subnormal or not finite stays, for the FP64 kernel.
+    {
+      uint32_t top = 0;  // high words of non-negative numbers compare like the numbers
+      for (int i = lane; i < K; i += 32) top = max(top, (uint32_t)__double2hiint(S.r[i]) & 0x7fffffffu);
+      const uint32_t e = __reduce_max_sync(0xffffffffu, top) >> 20;
+      const bool normal = e > 0 && e < 2046;
+      const double up = normal ? __hiloint2double((int)((2046 - e) << 20), 0) : 1.0;
+      for (int i = tid; i < K; i += G) {
+        const double f = S.r[i] * up;
+        S.F[i] = f;
+        S.rf[i] = (float)f;
+      }
+      if (tid == 0) S.down = normal ? __hiloint2double((int)(e << 20), 0) : 1.0;
+    }
     // ---- R, then M = R^-1 (a lane per column)
     if constexpr (W > 1 && K > 15) {  // most systems have fewer than 14 rows a lane
       if (n <= 32 * 14) factor<K, W, R, 14>(S, rows, n, h, lane);
@@ -747,7 +763,8 @@ __global__ void __launch_bounds__(W > 1 ? 32 * W : 128, MINB)
       if (tid == 0) a.status[s] = 3;
       continue;
     }
-    for (int i = tid; i < n; i += G) a.row_val[p0 + S.orig[i]] = S.wt[i] * S.t[i];  // s_hat = W t
+    const double down = S.down;
+    for (int i = tid; i < n; i += G) a.row_val[p0 + S.orig[i]] = S.wt[i] * S.t[i] * down;  // s_hat = W t
     if (tid == 0) a.status[s] = 0;
   }
 }

@@ -437,8 +437,9 @@ static cudaError_t launch_fold(const ApplyArgs<T>& a, const ApplyPlan& pl, cudaS
 template <typename T>
 static cudaError_t launch_template_pass(const ApplyArgs<T>& a, cudaStream_t s) {
   const ApplyPlan* pl = a.plan;
-  bool tma = pl && (sizeof(T) == 4 ? pl->tma32 : pl->tma64);
-  if (pl && pl->fold_act) {  // rows of phi whose length does not suit TMA are staged by plain copies
+  // a tensor map needs rows of phi that start and end at 16 bytes: the plan looks at their length, the address is the call's
+  const bool tma = pl && (sizeof(T) == 4 ? pl->tma32 : pl->tma64) && ((uintptr_t)a.phi & 15u) == 0;
+  if (pl && pl->fold_act) {  // what does not suit TMA is staged by plain copies
     if (pl->R == 3) return tma ? launch_fold<T, 3, true>(a, *pl, s) : launch_fold<T, 3, false>(a, *pl, s);
     return tma ? launch_fold<T, 2, true>(a, *pl, s) : launch_fold<T, 2, false>(a, *pl, s);
   }

@@ -80,7 +80,11 @@ __global__ void __launch_bounds__(256) k_apply_irregular(ApplyArgs<T> a) {
 // 100^3 grid take 56 us in FP32, and 17 us with W = 8 (FP64 at 160^3, 50000
 // rows: 131 and 55 us).  From SEG_MANY rows on, where there are warps enough,
 // the repeated index work costs more than it gives (FP32, 280000 rows: 91 and
-// 93 us; 1.15 M rows: 306 and 370 us).
+// 93 us; 1.15 M rows: 306 and 370 us; FP64 within 1 % either way, whole applies of 141^3 to 201^3).
+// 2-D in FP64 always takes one warp: the nine segments of a row have no chain to cut, and blocks with
+// shared memory of their own, beside the template pass's larger ones on few SMs, make applies that follow
+// one another wait for the SMs to change their partition: 29 us an apply at 200^2 to 300^2 with one warp, 110
+// to 140 us with eight (FP32, where both passes fit one partition: 13 us either way, and 24 instead of 27 us alone).
 constexpr int SEG_BLOCK_WARPS = 8;
 constexpr int64_t SEG_MANY = 262144;
 
@@ -112,6 +116,7 @@ __global__ void __launch_bounds__(32 * SEG_BLOCK_WARPS) k_apply_irregular_seg(Ap
     const int64_t stride = a.n_rows;
     const T* row = a.rows + a.irr_row[t];
     const int64_t ncell = a.ncell;
+    const T* cf = row;
 #pragma unroll 1
     for (int sgi = warp % W; sgi < NZ * NY; sgi += W) {
       const int dz = D == 3 ? sgi / NY - L : 0;
@@ -121,8 +126,11 @@ __global__ void __launch_bounds__(32 * SEG_BLOCK_WARPS) k_apply_irregular_seg(Ap
       const bool wide = !(az > R || ay > R);  // x extent L (wide) or R
       const int X = wide ? L : R;
       const int zz = cz + dz, yy = cy + dy;
-      if (zz < 0 || zz >= nz || yy < 0 || yy >= ny) continue;
-      const T* cf = row + (int64_t)seg_first<R, D>(dy, dz) * stride;
+      if (zz < 0 || zz >= nz || yy < 0 || yy >= ny) {
+        cf += (int64_t)(2 * X + 1) * stride;
+        continue;
+      }
+      if (W > 1) cf = row + (int64_t)seg_first<R, D>(dy, dz) * stride;  // one warp walks on from the last segment
       const int64_t base = (int64_t)nx * ((int64_t)yy + (int64_t)ny * zz) + cx;
       if (base - X >= 0 && base + X < ncell) {
         const T* ph = a.phi + base;
@@ -250,7 +258,8 @@ static cudaError_t launch_seg_w(const ApplyArgs<T>& a, cudaStream_t st) {
 
 template <typename T>
 static cudaError_t launch_seg(const ApplyArgs<T>& a, cudaStream_t st) {
-  return a.n_irr < SEG_MANY ? launch_seg_w<T, SEG_BLOCK_WARPS>(a, st) : launch_seg_w<T, 1>(a, st);
+  const bool shared = a.n_irr < SEG_MANY && !(sizeof(T) == 8 && a.plan->dim == 2);
+  return shared ? launch_seg_w<T, SEG_BLOCK_WARPS>(a, st) : launch_seg_w<T, 1>(a, st);
 }
 
 // class cells outside the runs and the slab bricks: per-cell segment walk over the canonical rows

@@ -1,0 +1,32 @@
+"""The operator's time on small FP64 grids, each against a case of the same run that cannot differ much from it.  In 2-D the
+passes of an apply take what one row's chain and one tile take until the grid fills the chip (29 us at 100^2 and at
+300^2): applies that follow one another on 300^2 take at most 2.5 times those on 100^2 (1.0; with eight warps to a row
+in FP64 it was 4.8, the SMs changing their shared memory's partition in turn)."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _time(dim, n, inside, dtype):
+    import torch
+    import paper_1411_4283_gb300 as P
+    c = (0.503, 0.497, 0.501)[:dim]
+    g = (P.eb_geometry_spheres if dim == 3 else P.eb_geometry_circles)(n, [c], [0.45 if inside else 0.3], inside=inside,
+                                                                     moment_degree=4)
+    st = P.eb_build_stencils(g, order=4)
+    x = torch.rand(n ** dim, device="cuda", dtype=getattr(torch, dtype))
+    y = torch.empty_like(x)
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    out = []
+    for _ in range(9):
+        ev[0].record()
+        for _ in range(40):
+            P.eb_apply(st, x, y)
+        ev[1].record()
+        ev[1].synchronize()
+        out.append(ev[0].elapsed_time(ev[1]))
+    return sorted(out)[4]
+
+
+def test_small_2d_grids_take_one_time():
+    assert _time(2, 300, False, "float64") <= 2.5 * _time(2, 100, False, "float64")

@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <stdint.h>
 #include <string.h>
+#include <vector>
 
 #include "eb_apply.cuh"
 #include "eb_internal.cuh"
@@ -416,7 +417,7 @@ static cudaError_t launch_fold(const ApplyArgs<T>& a, const ApplyPlan& pl, cudaS
   ta.nz = pl.nz;
   ta.ntx = (pl.nx + FD_OX - 1) / FD_OX;
   ta.nty = (pl.ny + FD_OY - 1) / FD_OY;
-  ta.zchunk = 8;
+  ta.zchunk = TMA ? 8 : pl.fold_zchunk[sizeof(T) == 8];
   ta.nzc = (pl.nz + ta.zchunk - 1) / ta.zchunk;
   ta.items = (int64_t)ta.ntx * ta.nty * ta.nzc;
   ta.kind = a.kind;
@@ -448,7 +449,7 @@ static cudaError_t launch_template_pass(const ApplyArgs<T>& a, cudaStream_t s) {
   const ApplyPlan* pl = a.plan;
   // a tensor map needs rows of phi that start and end at 16 bytes: the plan looks at their length, the address is the call's
   const bool tma = pl && (sizeof(T) == 4 ? pl->tma32 : pl->tma64) && ((uintptr_t)a.phi & 15u) == 0;
-  if (pl && pl->fold_act) {  // what does not suit TMA is staged by plain copies
+  if (pl && pl->fold_act && (tma || pl->fold_copies[sizeof(T) == 8])) {
     if (pl->R == 3) return tma ? launch_fold<T, 3, true>(a, *pl, s) : launch_fold<T, 3, false>(a, *pl, s);
     return tma ? launch_fold<T, 2, true>(a, *pl, s) : launch_fold<T, 2, false>(a, *pl, s);
   }
@@ -492,22 +493,22 @@ __global__ void __launch_bounds__(256) k_apply_transpose(ApplyArgs<T> a) {
   a.y[j] = acc;
 }
 
-// act[(z * 4 nty + g) * ntx + tx]: 1 when one of the cells (64 of x, FD_YB rows of y) of group g in tile column tx
-// of plane z has the template row; a warp per entry
+// act[(z * 4 nty + g) * ntx + tx]: how many of the cells (64 of x, FD_YB rows of y; up to 255) of group g in tile
+// column tx of plane z have the template row; a warp per entry
 __global__ void k_fold_active(const uint8_t* __restrict__ kind, int nx, int ny, int nz, int ntx, int ngy,
                               uint8_t* __restrict__ act) {
   const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (t >= (int64_t)nz * ngy * ntx) return;
   const int lane = threadIdx.x & 31;
   const int tx = (int)(t % ntx), g = (int)(t / ntx % ngy), z = (int)(t / ((int64_t)ntx * ngy));
-  bool any = false;
+  int cells = 0;
   for (int r = 0; r < FD_YB; ++r) {
     const int y = g * FD_YB + r;
     for (int x = tx * FD_OX + lane; y < ny && x < nx && x < (tx + 1) * FD_OX; x += 32)
-      any |= kind[x + (int64_t)nx * (y + (int64_t)ny * z)] == 1;
+      cells += kind[x + (int64_t)nx * (y + (int64_t)ny * z)] == 1;
   }
-  any = __any_sync(0xffffffffu, any);
-  if (lane == 0) act[t] = any;
+  cells = __reduce_add_sync(0xffffffffu, cells);
+  if (lane == 0) act[t] = (uint8_t)min(cells, 255);
 }
 int64_t fold_act_size(int nx, int ny, int nz) {
   return (int64_t)nz * ((ny + FD_OY - 1) / FD_OY * (FD_OY / FD_YB)) * ((nx + FD_OX - 1) / FD_OX);
@@ -518,6 +519,61 @@ cudaError_t fold_active(const uint8_t* kind, int nx, int ny, int nz, uint8_t* ac
                                                        (ny + FD_OY - 1) / FD_OY * (FD_OY / FD_YB), act);
   eb::count_launch();
   return cudaGetLastError();
+}
+
+// The folded pass with plain copies against the general template pass, for rows of phi that do not suit TMA.  The
+// general pass spreads its cells over the whole chip; the folded one does a quarter of the arithmetic, but a CTA per SM
+// works through pieces of tiles, and a small grid has few of them.  In FP64, where a plane of a tile takes 50 us
+// (R = 3; R = 2: 27 us), pieces of 8 planes left most SMs idle on grids up to 120^3 (inside a sphere at 41^3, R = 3: 328 us
+// an apply, 112 us with the general pass), so the pieces are as thin as it takes for the busiest CTA to have the
+// least to do, by the tiles' active row groups (0.2 of a plane for a piece's first planes, 0.05 for a plane's barriers);
+// with two rounds of CTAs or more the pieces stay at 8, where the sum is even enough (141^3: 1679 us, 1697 us with it).
+// The folded pass pays from FOLD_CELLS template cells for each plane of the busiest CTA's on (applies in us, general
+// and folded pass: R = 3, box minus a sphere, 45^3 with 6000 cells a plane 206 and 190, 53^3 with 15600 286 and 199, inside a sphere 47^3
+// with 13700 162 and 172, 53^3 with 20900 206 and 128; R = 2, box, 45^3 with 16600 99 and 96, alone 84 and 115, inside,
+// 47^3 with 18500 66 and 71, 65^3 with 24600 136 and 113).  In FP32 a plane takes 3 us and pieces of 8 are no
+// loss; the folded pass pays from 2^14 template cells on for R = 3 (inside, 47^3 with 14000 cells 35 and 56 us, 53^3 with
+// 23000 64 and 57; box, 45^3 with 6000 54 and 49) and from 2^16 on for R = 2 (inside, 47^3 with 19000 18 and 36, 59^3 with
+// 44000 24 and 28, 65^3 with 62000 31 and 28; box, 61^3 with 76000 42 and 40).
+constexpr double FOLD_CELLS[2] = {22000.0, 15000.0};  // R = 2, 3
+void fold_plan(ApplyPlan* pl, const uint8_t* act) {
+  constexpr int NG = FD_OY / FD_YB;
+  const int ntx = (pl->nx + FD_OX - 1) / FD_OX, nty = (pl->ny + FD_OY - 1) / FD_OY, nz = pl->nz;
+  // per tile: the work of the planes below z, in planes of four active groups and FD_PX columns
+  std::vector<double> below((size_t)ntx * nty * (nz + 1));
+  int64_t cells = 0;
+  for (int tx = 0; tx < ntx; ++tx)
+    for (int ty = 0; ty < nty; ++ty) {
+      double* w = below.data() + (size_t)(tx * nty + ty) * (nz + 1);
+      const double group = std::min(FD_PX, pl->nx - tx * FD_OX + 2 * TT_XH) / (double)(NG * FD_PX);
+      for (int z = 0; z < nz; ++z) {
+        w[z + 1] = w[z] + 0.05;
+        for (int g = 0; g < NG; ++g) {
+          const int n = act[((int64_t)z * nty * NG + ty * NG + g) * ntx + tx];
+          cells += n;
+          if (n > 0) w[z + 1] += group;
+        }
+      }
+    }
+  pl->fold_copies[0] = cells >= (pl->R == 3 ? 1 << 14 : 1 << 16);
+  double best = 0.0;  // planes of the busiest CTA
+  for (int zc = 8; zc >= 1; --zc) {
+    const int nzc = (nz + zc - 1) / zc;
+    const int64_t items = (int64_t)ntx * nty * nzc;
+    std::vector<double> load(pl->nsm, 0.0);  // CTA i takes the items i, i + nsm, ...
+    for (int64_t i = 0; i < items; ++i) {
+      const double* w = below.data() + (size_t)(i / nzc) * (nz + 1);
+      const int z0 = (int)(i % nzc) * zc;
+      load[i % pl->nsm] += 0.2 + w[std::min(z0 + zc, nz)] - w[z0];
+    }
+    const double most = *std::max_element(load.begin(), load.end());
+    if (zc == 8 || most < 0.95 * best) {
+      best = most;
+      pl->fold_zchunk[1] = zc;
+    }
+    if (zc == 8 && items >= 2 * pl->nsm) break;
+  }
+  pl->fold_copies[1] = cells >= FOLD_CELLS[pl->R == 3] * best;
 }
 
 template <typename T>

@@ -69,7 +69,10 @@ struct ApplyPlan {
   int fsym = 0;                  // template even in x, y and z (to a few ulps): fully folded pass (3-D)
   std::vector<float> fold32;     // T(a, b, c), a, b, c in 0..R+1: the mean of the cube's eight sign images
   std::vector<double> fold64;
-  uint8_t* fold_act = nullptr;   // which groups of rows of the folded pass's tiles hold template cells (null: not used)
+  uint8_t* fold_act = nullptr;   // template cells (up to 255) in the row groups of the folded pass's tiles (null: not used)
+  // where rows of phi do not suit TMA, in FP32 and FP64 (fold_plan): the folded pass staged by plain copies, else the
+  // general template pass; planes of a work item of the former
+  int fold_copies[2] = {0, 0}, fold_zchunk[2] = {8, 8};
   int32_t* err;                  // device error word (bounded waits)
   cudaStream_t side;             // irregular pass runs here, overlapped with the template pass
   cudaEvent_t fork, join;
@@ -79,6 +82,8 @@ struct ApplyPlan {
 // fold_act for the cell kinds (eb_apply_fold.cuh): its size and its values
 int64_t fold_act_size(int nx, int ny, int nz);
 cudaError_t fold_active(const uint8_t* kind, int nx, int ny, int nz, uint8_t* act, cudaStream_t s);
+// fold_copies and fold_zchunk from the values of fold_act
+void fold_plan(ApplyPlan* pl, const uint8_t* act);
 
 template <typename T>
 cudaError_t launch_apply(const ApplyArgs<T>& a, cudaStream_t s);

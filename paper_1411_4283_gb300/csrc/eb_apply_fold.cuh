@@ -31,7 +31,8 @@
 // where the length of a row of phi is not a multiple of 16 bytes, by
 // asynchronous copies of single values (before, the general template pass ran
 // there: FP32 132 us at 101^3 and 981 us at 201^3, 47 and 204 us now; FP64 779
-// and 694 us at 101^3).
+// and 694 us at 101^3).  Which of the two such a grid takes, and in pieces of how
+// many planes, is fold_plan's (eb_apply.cu).
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(FD_THREADS) k_apply_fold(const __grid_constant
     auto groups = [&](int z) {
       uint32_t m = 0;
 #pragma unroll
-      for (int g = 0; g < FD_OY / FD_YB; ++g) m |= (uint32_t)ap[z * zstride + g * a.ntx] << g;
+      for (int g = 0; g < FD_OY / FD_YB; ++g) m |= (uint32_t)(ap[z * zstride + g * a.ntx] != 0) << g;
       return m;
     };
     // plane zz by copies: the thread's column tid % FD_PX, every fourth row

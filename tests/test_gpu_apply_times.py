@@ -1,7 +1,8 @@
 """The operator's time on small FP64 grids, each against a case of the same run that cannot differ much from it.  In 2-D the
 passes of an apply take what one row's chain and one tile take until the grid fills the chip (29 us at 100^2 and at
 300^2): applies that follow one another on 300^2 take at most 2.5 times those on 100^2 (1.0; with eight warps to a row
-in FP64 it was 4.8, the SMs changing their shared memory's partition in turn)."""
+in FP64 it was 4.8, the SMs changing their shared memory's partition in turn).  On a small ragged 3-D grid inside
+a sphere FP64 takes up to four times FP32 (2.2; the folded pass in pieces of eight planes took 6.9)."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -30,3 +31,7 @@ def _time(dim, n, inside, dtype):
 
 def test_small_2d_grids_take_one_time():
     assert _time(2, 300, False, "float64") <= 2.5 * _time(2, 100, False, "float64")
+
+
+def test_small_ragged_grid_in_fp64():
+    assert _time(3, 29, True, "float64") <= 4.0 * _time(3, 29, True, "float32")

@@ -1646,11 +1646,13 @@ static eb_status build_post(BuildCtx& c) {
     pl->seg = dm.nbr_box;
     if (ok && D == 3 && pl->fsym && (R == 2 || R == 3)) {
       EB_TRY(dalloc(st, &pl->fold_act, fold_act_size(pl->nx, pl->ny, pl->nz)));
-      EB_CUDA(fold_active(st->cell_kind, pl->nx, pl->ny, pl->nz, pl->fold_act, s));
-      std::vector<uint8_t> act(fold_act_size(pl->nx, pl->ny, pl->nz));
-      EB_CUDA(cudaMemcpyAsync(act.data(), pl->fold_act, act.size(), cudaMemcpyDeviceToHost, s));
+      std::vector<uint8_t> cells(fold_act_size(pl->nx, pl->ny, pl->nz));
+      uint8_t* dcells;
+      EB_TRY(tmp.get(&dcells, cells.size()));
+      EB_CUDA(fold_active(st->cell_kind, pl->nx, pl->ny, pl->nz, pl->fold_act, dcells, s));
+      EB_CUDA(cudaMemcpyAsync(cells.data(), dcells, cells.size(), cudaMemcpyDeviceToHost, s));
       EB_CUDA(cudaStreamSynchronize(s));
-      fold_plan(pl, act.data());
+      fold_plan(pl, cells.data());
     }
     if (pl->seg && D == 3 && (R == 2 || R == 3) && st->n_irr > 0) EB_TRY(build_quad_plan(st, pl, R, s, tmp));
     EB_CUDA(cudaStreamCreateWithFlags(&pl->side, cudaStreamNonBlocking));

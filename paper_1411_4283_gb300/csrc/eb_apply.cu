@@ -493,10 +493,10 @@ __global__ void __launch_bounds__(256) k_apply_transpose(ApplyArgs<T> a) {
   a.y[j] = acc;
 }
 
-// act[(z * 4 nty + g) * ntx + tx]: how many of the cells (64 of x, FD_YB rows of y; up to 255) of group g in tile
-// column tx of plane z have the template row; a warp per entry
+// act[(z * 4 nty + g) * ntx + tx]: 1 when one of the cells (64 of x, FD_YB rows of y) of group g in tile column tx
+// of plane z has the template row; ncells: how many (up to 255); a warp per entry
 __global__ void k_fold_active(const uint8_t* __restrict__ kind, int nx, int ny, int nz, int ntx, int ngy,
-                              uint8_t* __restrict__ act) {
+                              uint8_t* __restrict__ act, uint8_t* __restrict__ ncells) {
   const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (t >= (int64_t)nz * ngy * ntx) return;
   const int lane = threadIdx.x & 31;
@@ -508,15 +508,18 @@ __global__ void k_fold_active(const uint8_t* __restrict__ kind, int nx, int ny, 
       cells += kind[x + (int64_t)nx * (y + (int64_t)ny * z)] == 1;
   }
   cells = __reduce_add_sync(0xffffffffu, cells);
-  if (lane == 0) act[t] = (uint8_t)min(cells, 255);
+  if (lane == 0) {
+    act[t] = cells > 0;
+    ncells[t] = (uint8_t)min(cells, 255);
+  }
 }
 int64_t fold_act_size(int nx, int ny, int nz) {
   return (int64_t)nz * ((ny + FD_OY - 1) / FD_OY * (FD_OY / FD_YB)) * ((nx + FD_OX - 1) / FD_OX);
 }
-cudaError_t fold_active(const uint8_t* kind, int nx, int ny, int nz, uint8_t* act, cudaStream_t s) {
+cudaError_t fold_active(const uint8_t* kind, int nx, int ny, int nz, uint8_t* act, uint8_t* cells, cudaStream_t s) {
   const int64_t n = fold_act_size(nx, ny, nz);
   k_fold_active<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(kind, nx, ny, nz, (nx + FD_OX - 1) / FD_OX,
-                                                       (ny + FD_OY - 1) / FD_OY * (FD_OY / FD_YB), act);
+                                                       (ny + FD_OY - 1) / FD_OY * (FD_OY / FD_YB), act, cells);
   eb::count_launch();
   return cudaGetLastError();
 }
@@ -536,7 +539,7 @@ cudaError_t fold_active(const uint8_t* kind, int nx, int ny, int nz, uint8_t* ac
 // 23000 64 and 57; box, 45^3 with 6000 54 and 49) and from 2^16 on for R = 2 (inside, 47^3 with 19000 18 and 36, 59^3 with
 // 44000 24 and 28, 65^3 with 62000 31 and 28; box, 61^3 with 76000 42 and 40).
 constexpr double FOLD_CELLS[2] = {22000.0, 15000.0};  // R = 2, 3
-void fold_plan(ApplyPlan* pl, const uint8_t* act) {
+void fold_plan(ApplyPlan* pl, const uint8_t* ncells) {
   constexpr int NG = FD_OY / FD_YB;
   const int ntx = (pl->nx + FD_OX - 1) / FD_OX, nty = (pl->ny + FD_OY - 1) / FD_OY, nz = pl->nz;
   // per tile: the work of the planes below z, in planes of four active groups and FD_PX columns
@@ -549,7 +552,7 @@ void fold_plan(ApplyPlan* pl, const uint8_t* act) {
       for (int z = 0; z < nz; ++z) {
         w[z + 1] = w[z] + 0.05;
         for (int g = 0; g < NG; ++g) {
-          const int n = act[((int64_t)z * nty * NG + ty * NG + g) * ntx + tx];
+          const int n = ncells[((int64_t)z * nty * NG + ty * NG + g) * ntx + tx];
           cells += n;
           if (n > 0) w[z + 1] += group;
         }

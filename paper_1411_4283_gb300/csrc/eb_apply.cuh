@@ -69,7 +69,7 @@ struct ApplyPlan {
   int fsym = 0;                  // template even in x, y and z (to a few ulps): fully folded pass (3-D)
   std::vector<float> fold32;     // T(a, b, c), a, b, c in 0..R+1: the mean of the cube's eight sign images
   std::vector<double> fold64;
-  uint8_t* fold_act = nullptr;   // template cells (up to 255) in the row groups of the folded pass's tiles (null: not used)
+  uint8_t* fold_act = nullptr;   // which groups of rows of the folded pass's tiles hold template cells (null: not used)
   // where rows of phi do not suit TMA, in FP32 and FP64 (fold_plan): the folded pass staged by plain copies, else the
   // general template pass; planes of a work item of the former
   int fold_copies[2] = {0, 0}, fold_zchunk[2] = {8, 8};
@@ -79,11 +79,11 @@ struct ApplyPlan {
   int nsm;
 };
 
-// fold_act for the cell kinds (eb_apply_fold.cuh): its size and its values
+// fold_act for the cell kinds (eb_apply_fold.cuh): its size, its values and the template cells (up to 255) of each entry
 int64_t fold_act_size(int nx, int ny, int nz);
-cudaError_t fold_active(const uint8_t* kind, int nx, int ny, int nz, uint8_t* act, cudaStream_t s);
-// fold_copies and fold_zchunk from the values of fold_act
-void fold_plan(ApplyPlan* pl, const uint8_t* act);
+cudaError_t fold_active(const uint8_t* kind, int nx, int ny, int nz, uint8_t* act, uint8_t* cells, cudaStream_t s);
+// fold_copies and fold_zchunk from the entries' template cells
+void fold_plan(ApplyPlan* pl, const uint8_t* cells);
 
 template <typename T>
 cudaError_t launch_apply(const ApplyArgs<T>& a, cudaStream_t s);

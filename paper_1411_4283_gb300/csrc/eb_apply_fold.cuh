@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(FD_THREADS) k_apply_fold(const __grid_constant
     auto groups = [&](int z) {
       uint32_t m = 0;
 #pragma unroll
-      for (int g = 0; g < FD_OY / FD_YB; ++g) m |= (uint32_t)(ap[z * zstride + g * a.ntx] != 0) << g;
+      for (int g = 0; g < FD_OY / FD_YB; ++g) m |= (uint32_t)ap[z * zstride + g * a.ntx] << g;
       return m;
     };
     // plane zz by copies: the thread's column tid % FD_PX, every fourth row

@@ -1316,8 +1316,8 @@ static eb_status build_post(BuildCtx& c) {
   {
     // counted on the device: face states and system statuses (4: left by the mixed path, solved in FP64)
     unsigned long long* counts;
-    unsigned long long hc[5];
-    EB_TRY(tmp.get(&counts, 5));
+    unsigned long long hc[4];
+    EB_TRY(tmp.get(&counts, 4));
     EB_CUDA(cudaMemsetAsync(counts, 0, sizeof(hc), s));
     for (int d = 0; d < D; ++d) {
       EB_CUDA(count_faces(st->face_slot[d], dm.nface[d], n_unique, counts, s));
@@ -1329,11 +1329,9 @@ static eb_status build_post(BuildCtx& c) {
     EB_CUDA(cudaStreamSynchronize(s));
     info->n_flux_faces = (int64_t)hc[0] + nc;
     info->n_class_faces = (int64_t)hc[1];
-    info->n_ls_fp64 = c.P.ls_precision == EB_LS_FP64 ? n_slots : (int64_t)hc[4];
+    info->n_ls_fp64 = c.P.ls_precision == EB_LS_FP64 ? n_slots : (int64_t)hc[3];
     info->ls_fp64_flops = c.ls_flops[0];
     info->ls_fp32_flops = c.ls_flops[1];
-    const bool unbuilt = hc[3] > 0;  // a row flagged by the row builder
-    if (unbuilt) { set_error("an LS row could not be built"); return EB_ERR_INVALID; }
     if (hc[2] > 0) {
       std::vector<int32_t> hs(n_slots);
       EB_CUDA(cudaMemcpyAsync(hs.data(), status, n_slots * 4, cudaMemcpyDeviceToHost, s));

@@ -399,7 +399,7 @@ __device__ void shift_moments(const Tables& T, const double* __restrict__ in, co
 // and weight recorded in row[0..4], so that the warp can shift all pending rows of a chunk with
 // every lane busy (row_finish).  Wall rows over a cut face are shifted here.
 __device__ double row_prepare(const LsArgs& a, const Tables& T, uint32_t desc, const int* base, const double* x0s,
-                              double* row, int* bad, int* pend) {
+                              double* row, int* pend) {
   const Dims& dm = a.dm;
   const int K = T.K;
   *pend = 0;
@@ -646,7 +646,6 @@ __global__ void __launch_bounds__(LS_SYS * LS_NW * 32, 1)
       face_xyz(dm, dface, flocal, base);
       x0s[dface] = -0.5;
     }
-    int bad = 0;
     for (int i = lane + 32 * h; i < K * K; i += 32 * LS_NW) S.R[i] = 0.0;
     // ---- row-streamed Householder QR of B = W A: R accumulates the triangular factor
     for (int c0 = 0; c0 < n; c0 += CH) {
@@ -665,7 +664,7 @@ __global__ void __launch_bounds__(LS_SYS * LS_NW * 32, 1)
         double* dst = row_at(li);
         int pd = 0;
         if (i < n) {
-          scr_w[i] = row_prepare(a, T, a.row_desc[p0 + i], base, x0s, dst, &bad, &pd);
+          scr_w[i] = row_prepare(a, T, a.row_desc[p0 + i], base, x0s, dst, &pd);
         } else {
           for (int k = 0; k < K; ++k) dst[k] = 0.0;
         }
@@ -1122,14 +1121,13 @@ __global__ void k_count_faces(const int32_t* __restrict__ slot, int64_t n, int64
   }
 }
 __global__ void k_count_status(const int32_t* __restrict__ status, int64_t n, unsigned long long* __restrict__ counts) {
-  unsigned c[3] = {0, 0, 0};
+  unsigned c[2] = {0, 0};
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t v = status[i];
     c[0] += v == 1;
-    c[1] += v == 2;
-    c[2] += v == 4;
+    c[1] += v == 4;
   }
-  for (int k = 0; k < 3; ++k) {
+  for (int k = 0; k < 2; ++k) {
     c[k] = __reduce_add_sync(0xffffffffu, c[k]);
     if ((threadIdx.x & 31) == 0 && c[k]) atomicAdd(counts + 2 + k, (unsigned long long)c[k]);
   }

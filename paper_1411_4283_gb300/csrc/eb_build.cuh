@@ -92,7 +92,7 @@ struct LsArgs {
   int64_t n_slots;
   const int32_t* slot_list;  // [n_slots] systems to solve (null: 0 .. n_slots-1)
   int32_t* next;       // work counter
-  int32_t* status;     // [n_slots]: 0 ok, 1 rank deficient, 2 unsupported row, 3 left to the FP64 path
+  int32_t* status;     // [n_slots]: 0 ok, 1 rank deficient, 3 left to the FP64 path, 4 solved there
   double* scratch;     // per system in flight: LS_SCRATCH doubles (FP64), see k_lsq_mixed (mixed)
   int32_t* err;        // set when a bounded wait between the two warps of a system gives up
   double* flops;       // [2] executed flops, accumulated: FP64, FP32
@@ -172,8 +172,8 @@ __global__ void k_assemble_rows(AsmArgs a, const int32_t* rep_cell, int64_t nrep
 // boundary entries of the irregular cells' rows: counted into cnt (bptr null) or written
 cudaError_t assemble_b_launch(const AsmArgs& a, const int32_t* cells, int64_t ncells, int64_t* cnt, const int64_t* bptr,
                               int64_t* bcol, double* bval, cudaStream_t s);
-// counts[0, 1] += the faces of one direction with a slot and with a class slot; counts[2..4] += the systems of
-// status 1 (rank deficient), 2 (a row that could not be built) and 4 (solved by the FP64 pass)
+// counts[0, 1] += the faces of one direction with a slot and with a class slot; counts[2, 3] += the systems of
+// status 1 (rank deficient) and 4 (solved by the FP64 pass)
 cudaError_t count_faces(const int32_t* slot, int64_t n, int64_t n_unique, unsigned long long* counts, cudaStream_t s);
 cudaError_t count_status(const int32_t* status, int64_t n, unsigned long long* counts, cudaStream_t s);
 

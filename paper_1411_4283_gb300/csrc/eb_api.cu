@@ -1760,7 +1760,7 @@ eb_status eb_bc_rhs(const eb_stencils* st, const double* g_eb, const double* g_w
   if ((st->dm.n_cut > 0 && !g_eb) || (st->n_wall > 0 && !g_wall)) { set_error("missing boundary data"); return EB_ERR_INVALID; }
   cudaStream_t s = (cudaStream_t)stream;
   EB_CUDA(vec_fill64(st->dm.ncell, Bg, 0.0, s));
-  EB_CUDA(launch_bg(st->n_irr, st->irr_cell, st->b_ptr, st->b_col, st->b_val, st->dm.n_grid_faces, st->b_wpos, g_eb,
+  EB_CUDA(launch_bg(st->dm.dim, st->n_irr, st->irr_cell, st->b_ptr, st->b_col, st->b_val, st->dm.n_grid_faces, st->b_wpos, g_eb,
                     g_wall, st->inv_kappa, kappa_weighted, Bg, s));
   return EB_OK;
 }

@@ -122,24 +122,30 @@ __global__ void k_norms(int64_t n, const uint8_t* flag, const double* kappa, con
   }
 }
 
-// B g (kappa-weighted B, CSR over irregular cells)
+// B g (kappa-weighted B, CSR over irregular cells), G lanes per row.  A thread per row left the loads uncoalesced and the
+// longest row's chain as the kernel's time (0.53 ms at 48^3, 0.11 ms with a warp per row): a 3-D row has tens to
+// hundreds of entries.  A 2-D row has ten to forty, and where there are more rows than warps on the chip (9728) a warp for
+// each leaves its lanes idle: 65 us at 4096^2 in second order, a thread per row 50 us, eight lanes 42 us (fourth order
+// at 1024^2 21.5, 23.3 and 15.2 us); with fewer rows the warp's shorter chain is the better one (a residual on 32^2,
+// the operator and this: 38 us, 41 us with eight lanes).
+constexpr int64_t BG_WARPS = 8192;
+template <int G>
 __global__ void k_bg(int64_t n_irr, const int32_t* irr_cell, const int64_t* bptr, const int64_t* bcol,
                      const double* bval, int64_t n_grid_faces, const int64_t* wall_pos, const double* g_eb,
                      const double* g_wall, const double* inv_kappa, int kw, double* out) {
-  // a warp per row (a few to some hundred entries); a thread per row left the loads uncoalesced and the longest
-  // row's chain as the kernel's time: 0.53 ms at 48^3, 0.11 ms now
-  const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (t >= n_irr) return;
-  const int lane = threadIdx.x & 31;
+  const int64_t row = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
+  if (row - threadIdx.x % 32 / G >= n_irr) return;  // a whole warp
+  const int64_t t = G == 32 ? row : min(row, n_irr - 1);  // the last warp's other groups repeat the last row
+  const int lane = threadIdx.x % G;
   double acc = 0.0;
-  for (int64_t k = bptr[t] + lane; k < bptr[t + 1]; k += 32) {
+  for (int64_t k = bptr[t] + lane; k < bptr[t + 1]; k += G) {
     int64_t col = bcol[k];
     double g = col >= n_grid_faces ? g_eb[col - n_grid_faces] : g_wall[wall_pos[k]];
     acc += bval[k] * g;
   }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   int64_t c = irr_cell[t];
-  if (lane == 0) out[c] = kw ? acc : acc * inv_kappa[c];
+  if (lane == 0 && (G == 32 || row < n_irr)) out[c] = kw ? acc : acc * inv_kappa[c];
 }
 
 static unsigned grid_for(int64_t n) {
@@ -161,12 +167,15 @@ cudaError_t compute_rhs(int64_t n, const uint8_t* flag, const double* kappa, con
   return cudaGetLastError();
 }
 
-cudaError_t launch_bg(int64_t n_irr, const int32_t* irr_cell, const int64_t* bptr, const int64_t* bcol,
+cudaError_t launch_bg(int dim, int64_t n_irr, const int32_t* irr_cell, const int64_t* bptr, const int64_t* bcol,
                       const double* bval, int64_t n_grid_faces, const int64_t* wall_pos, const double* g_eb,
                       const double* g_wall, const double* inv_kappa, int kw, double* out, cudaStream_t s) {
   if (n_irr == 0) return cudaSuccess;
-  k_bg<<<(unsigned)((n_irr + 7) / 8), 256, 0, s>>>(n_irr, irr_cell, bptr, bcol, bval, n_grid_faces, wall_pos,
-                                                       g_eb, g_wall, inv_kappa, kw, out); eb::count_launch();
+  const bool few = dim == 2 && n_irr > BG_WARPS;
+  const int lanes = few ? 8 : 32;
+  const auto kern = few ? k_bg<8> : k_bg<32>;
+  kern<<<(unsigned)((n_irr * lanes + 255) / 256), 256, 0, s>>>(n_irr, irr_cell, bptr, bcol, bval, n_grid_faces, wall_pos,
+                                                               g_eb, g_wall, inv_kappa, kw, out); eb::count_launch();
   return cudaGetLastError();
 }
 

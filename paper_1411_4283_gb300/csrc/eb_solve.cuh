@@ -12,7 +12,7 @@ namespace eb {
 cudaError_t vec_fill64(int64_t n, double* x, double v, cudaStream_t s);
 cudaError_t compute_rhs(int64_t n, const uint8_t* flag, const double* kappa, const double* rho, const double* bg,
                         double* out, cudaStream_t s);
-cudaError_t launch_bg(int64_t n_irr, const int32_t* irr_cell, const int64_t* bptr, const int64_t* bcol,
+cudaError_t launch_bg(int dim, int64_t n_irr, const int32_t* irr_cell, const int64_t* bptr, const int64_t* bcol,
                       const double* bval, int64_t n_grid_faces, const int64_t* wall_pos, const double* g_eb,
                       const double* g_wall, const double* inv_kappa, int kw, double* out, cudaStream_t s);
 cudaError_t launch_norms(int64_t n, const uint8_t* flag, const double* kappa, const double* e, double* out,

@@ -23,10 +23,14 @@
 // the shifts of the rows that need one; FP32 products are 64 times cheaper on this part, which pays for 11 of
 // them in place of one DFMA.  As it stands the FP64 pipe is 40 % busy and the rest is the latency of the serial
 // parts (factor 27 %, row lists and shifts 25 % of a block's time) that two blocks per SM do not hide: the matrix
-// in registers takes 255 of them, and three blocks with the spills that costs measured the same.  90,201 systems
-// of the 48^3 box minus a sphere (n = 396 on average, K = 35): 22.2 ms; the kernel before it (FP32 Householder
-// with the chunk in shared memory, FP64 corrections: 4 n K (1 + 3.1) FP64 flops, 35 lanes of 64 in B^T t) 71.3 ms.
-// Error of the operator against the FP64 kernel's at 63^3: 1.0e-14 (before 2.0e-14).
+// in registers takes all 255 of them and spills 528 bytes a thread as it is (the batch form 600), and three blocks, with
+// more spills, measured the same.  90,201 systems of the 48^3 box minus a sphere (n = 396 on average, K = 35): 22.4 ms;
+// the kernel before it (FP32 Householder with the chunk in shared memory, FP64 corrections: 4 n K (1 + 3.1) FP64 flops,
+// 35 lanes of 64 in B^T t) 71.3 ms.
+// Error against 64 bits on the same moment tables (2-norm of operator and boundary part on rough data), in brackets
+// of the kernel before and of the FP64 kernel: 63^3 box minus a sphere 4.1e-15 and 1.2e-14 (6.4e-15 and 2.6e-14; 3.2e-15
+// and 1.1e-14), Neumann data inside a sphere at 60^3 1.35e-15 and 1.17e-13 (1.32e-15 and 1.16e-13; 1.44e-15 and
+// 1.17e-13), second order at 97^3 6.2e-16 and 2.9e-15 (1.0e-15 and 5.5e-15; 7.0e-16 and 2.9e-15).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -775,8 +779,10 @@ __global__ void __launch_bounds__(W > 1 ? 32 * W : 128, MINB)
 // A warp per system while 32 R rows hold the largest one (2-D and second order: 4 systems a block, no block
 // barriers), else a block of four warps per system, whose lanes hold any system's rows (MAXROWS / 32 = 20).
 // Both on the same systems: 3-D second order at 80^3 4.64 ms by warps and 7.19 ms by blocks, 2-D fourth order at
-// 512^2 (9328 faces) 0.21 and 0.52 ms.  Fourth order in 3-D needs the registers of four warps for one system's rows;
-// at 128^3 two blocks an SM take 133.7 ms, three (with spills) 132.0 ms, seven warps a system 140.7 ms.
+// 512^2 (9328 faces) 0.21 and 0.52 ms.  One large system takes a whole build, or batch, to the block shape, which is
+// still well below the kernel before: second order with R_n = 3, 2-D at 512^2 (71 rows) 0.29 ms (before 0.76), 3-D at
+// 80^3 (468 rows) 16.3 ms (87.8).  Fourth order in 3-D needs the registers of four warps for one system's rows;
+// at 128^3 two blocks an SM take 133.7 ms, three (with more spills) 132.0 ms, seven warps a system 140.7 ms.
 namespace {
 
 struct MixShape {

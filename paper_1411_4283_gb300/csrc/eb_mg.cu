@@ -215,9 +215,11 @@ struct MgSweep {
 //   MG_FIRST, MG_PROLONG   no sweep: the first one from x = 0, out = w b / diag; x + x_c (piecewise constant on volumes)
 //   MG_PRE, MG_POST        those values and the sweep that follows, in one pass
 // The fused passes repeat a division or two more loads for each neighbour: 6.9 and 7.1 us at 64^3 in FP32 (4.8
-// for the sweep alone, before another pass and its launch), but 29 and 30 us at 128^3 (two passes: 25 and 26 us), hence the line between them; in FP64
-// the divide is a sequence on a pipe 64 times slower and the line lies lower.  The passes of a cycle at 128^3 took
-// 225 us in 18 launches before, 136 us in 14 now.
+// for the sweep alone, before another pass and its launch), but 29 and 30 us at 128^3 (two passes: 25 and 26 us), hence the line between them.  In FP64
+// the divide is a sequence on a pipe 64 times slower: an iteration of an FP64 solve takes 734 us in two passes and 741 us
+// fused at 30^3, 1071 and 1090 at 40^3, 1271 and 1304 at 48^3, 2093 and 2243 at 80^3, 4201 and 4734 at 128^3, so the line lies
+// where the two are within 2 %.  The level passes of a cycle at 128^3 in FP32 took 225 us in 18 launches before and
+// take 133 us in 14 now, k_mg_coarse 85 and 32 us.
 enum { MG_PLAIN, MG_FIRST, MG_PROLONG, MG_PRE, MG_POST };
 template <typename T>
 constexpr int64_t MG_FUSE_CELLS = sizeof(T) == 4 ? 1 << 20 : 1 << 16;

